@@ -448,6 +448,24 @@ kpm_status kpm_batch_set_staged(kpm_batch b, int staged);
  * the current traversal chunk (any output may be NULL). */
 kpm_status kpm_batch_get_staged(kpm_batch b, int* staged, int* tile_rows, int* stages);
 
+/* Column-strip form (columns = 1; what a batch starts with where it applies):
+ * the instances' vector columns as independent tasks of one persistent
+ * launch, each task running all products (Eq. (rn)) of a few columns of one
+ * instance with v_n in the shared memory of a CTA, or of a cluster of CTAs
+ * that hold a band of rows each, and v_{n-1} in registers.  2D and 3D
+ * stencils of uniform real hopping whose columns fit a cluster of 16 CTAs
+ * (KPM_EINVAL otherwise).  The products are the other forms' bit for bit and
+ * the moment dots sum the same terms in another order; an instance's moments
+ * depend only on the cluster size, which kpm_batch_info reports, and the
+ * instance.  Calls that set part of another form's configuration
+ * (kpm_batch_set_config, _set_rtiles, _set_chunk_bytes, _set_resident,
+ * _set_staged) leave it for that form; columns = 0 for the global-memory
+ * form with its defaults. */
+kpm_status kpm_batch_set_columns(kpm_batch b, int columns);
+
+/* Whether the column-strip form is set. */
+kpm_status kpm_batch_get_columns(kpm_batch b, int* columns);
+
 /* Current R-tiles, the number of instances tiled, and the largest R-tiles
  * this batch admits (min(4, G)). */
 kpm_status kpm_batch_get_rtiles(kpm_batch b, int* rtiles, int* top, int* max_rtiles);

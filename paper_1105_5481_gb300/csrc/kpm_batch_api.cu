@@ -16,11 +16,12 @@
 #include <vector>
 
 #include "kpm_batch.cuh"
+#include "kpm_cols.h"
 
 using namespace kpm;
 
 namespace {
-constexpr int FORM_GLOBAL = 0, FORM_RESIDENT = 1, FORM_STAGED = 2;
+constexpr int FORM_GLOBAL = 0, FORM_RESIDENT = 1, FORM_STAGED = 2, FORM_COLS = 3;
 }
 
 struct BatchConfig {
@@ -30,7 +31,8 @@ struct BatchConfig {
   int rtiles = 1;     // column tiles of a tiled instance (divides the chunks per row)
   int top = 0;        // the `top` instances of largest work are tiled (<= 0: all)
   int res = 0;        // vector rows: 0 global memory, 1 resident in the clusters' shared
-                      // memory, 2 staged through shared-memory rings (chunk: tile size)
+                      // memory, 2 staged through shared-memory rings (chunk: tile size),
+                      // 3 column strips (kpm_cols.cuh; C its cluster size, chunk unused)
   int tpr = 1;        // threads per row relative to the 32-byte chunk (2: 16-byte chunks)
 };
 
@@ -49,7 +51,14 @@ struct kpm_batch_s {
   std::vector<BatchTask> inst_tasks; // one untiled task per instance (instance order)
   std::vector<BatchTask> host_tasks; // task slot order of the current configuration
   BatchTask* d_tasks = nullptr;
-  int* d_queue = nullptr;            // [0] task queue, [1 + i] tiles finished of instance i
+  // [0] task queue, [1 + i] tiles finished of instance i, [1 + count + i] its
+  // divergence flag (column-strip form)
+  int* d_queue = nullptr;
+
+  // column-strip form: its tasks and the scratch of its CTA partials
+  ColsTask* d_ctasks = nullptr;
+  double* d_cpart = nullptr;
+  size_t ctasks_cap = 0, cpart_cap = 0;
   void* d_pool = nullptr;            // vectors, sums, per-vector moments, operators
   double* d_mu = nullptr;            // [mu_total] in instance order (inside the pool)
   StepArgs proto{};                  // template-selecting prototype (first instance)
@@ -166,7 +175,119 @@ int max_clusters_stg(kpm_batch_s* b, const BatchConfig& c) {
                  : max_clusters_batch_stg_f64(b->cplx, a, c.C, sh.Tl, sh.Sl, sh.SWl);
 }
 
+// Whether the column-strip form can run the batch's operators: 2D and 3D
+// stencils with a uniform real hopping.
+bool cols_kind(const kpm_batch_s* b) {
+  const kpm_handle_s* h = b->handles[0];
+  return h->stencil && !b->cplx && !h->has_hop && (h->geom.dims == 2 || h->geom.dims == 3);
+}
+
+// The tasks of the column-strip form at cluster size C (false: some instance
+// does not fit), longest first; *us the estimated time of the batch.  Columns
+// are packed as many to a task as a CTA holds; where that leaves clusters
+// without work the tasks are made narrower (a column's moments do not depend
+// on the other columns of its task).
+struct ColsPlan {
+  std::vector<ColsTask> tasks;
+  size_t smem = 0, part = 0;
+  int clusters = 0;
+  double us = 0.0;
+};
+bool plan_cols(const kpm_batch_s* b, int C, ColsPlan* out) {
+  const kpm_handle_s* h0 = b->handles[0];
+  const bool ds = h0->has_onsite;
+  std::vector<ColsShape> shp(b->count);
+  size_t smem1 = 0;
+  for (int i = 0; i < b->count; ++i) {
+    const kpm_handle_s* h = b->handles[i];
+    if (!cols_shape(h->geom, h->n, b->R, b->fp32, C, &shp[i])) return false;
+    smem1 = std::max(smem1, cols_smem(shp[i], b->fp32, 1));
+  }
+  const int nclu = cols_max_clusters(b->fp32, h0->geom.dims, ds, C, smem1);
+  if (nclu < 1) return false;
+  auto width = [&](int i, int cap) { return std::max(1, std::min({b->R, shp[i].max_cols, cap})); };
+  int cap = b->R;
+  for (; cap > 1; cap = (cap + 1) / 2) {
+    int64_t n = 0;
+    for (int i = 0; i < b->count; ++i) n += (b->R + width(i, cap) - 1) / width(i, cap);
+    if (n >= 2 * (int64_t)nclu) break;
+  }
+  struct Item {
+    double us;
+    ColsTask t;
+  };
+  std::vector<Item> items;
+  ColsPlan p;
+  double total = 0.0;
+  for (int i = 0; i < b->count; ++i) {
+    const BatchTask& bt = b->inst_tasks[i];
+    const ColsShape& s = shp[i];
+    const int groups = (b->R + width(i, cap) - 1) / width(i, cap);
+    for (int g = 0; g < groups; ++g) {
+      const int c0 = (int)((int64_t)b->R * g / groups), c1 = (int)((int64_t)b->R * (g + 1) / groups);
+      ColsTask t{};
+      t.geom = bt.a.geom;
+      t.n = bt.a.n;
+      t.sc = bt.a.sc;
+      t.ds = bt.a.ds;
+      t.v[0] = bt.v[0];
+      t.v[1] = bt.v[1];
+      t.sums = bt.sums;
+      t.seed = bt.seed;
+      t.s = bt.realisation;
+      t.Rp = bt.a.Rp;
+      t.R = bt.R;
+      t.M = bt.M;
+      cols_set_layout(t, s, b->fp32, c0, c1 - c0);
+      t.n0 = 0;
+      t.n1 = bt.M / 2;
+      t.per_vec = bt.per_vec;
+      t.mu = bt.mu;
+      t.flags = b->d_queue + 1 + b->count + i;
+      t.tiles_done = b->d_queue + 1 + i;
+      t.ntiles = groups;
+      const double us = t.n1 * (s.us_fixed + t.ncol * s.us_col);
+      total += us;
+      p.us = std::max(p.us, us);
+      p.smem = std::max(p.smem, cols_smem(s, b->fp32, t.ncol));
+      items.push_back({us, t});
+    }
+  }
+  std::stable_sort(items.begin(), items.end(), [](const Item& x, const Item& y) { return x.us > y.us; });
+  for (Item& it : items) {
+    if (C > 1) {
+      it.t.part = (double*)(p.part * sizeof(double));  // offset, made a pointer when the scratch exists
+      p.part += (size_t)C * it.t.n1 * 2 * it.t.ncol;
+    }
+    p.tasks.push_back(it.t);
+  }
+  p.clusters = std::min((int)p.tasks.size(), cols_max_clusters(b->fp32, h0->geom.dims, ds, C, p.smem));
+  if (p.clusters < 1) return false;
+  p.us = std::max(p.us, total / p.clusters);
+  *out = std::move(p);
+  return true;
+}
+
+// The cluster size of least estimated time (0: the form does not apply).
+int cols_cluster(const kpm_batch_s* b) {
+  if (!cols_kind(b)) return 0;
+  int best = 0;
+  double best_us = 1e300;
+  for (int C : {1, 2, 4, 8, 16}) {
+    ColsPlan p;
+    if (plan_cols(b, C, &p) && p.us < best_us) {
+      best_us = p.us;
+      best = C;
+    }
+  }
+  return best;
+}
+
 int cfg_clusters(kpm_batch_s* b, const BatchConfig& c) {
+  if (c.res == FORM_COLS) {
+    ColsPlan p;
+    return cols_kind(b) && plan_cols(b, c.C, &p) ? p.clusters : 0;
+  }
   if (c.res == FORM_STAGED) return max_clusters_stg(b, c);
   return c.res ? max_clusters_res(b, c.C) : max_clusters(b, c);
 }
@@ -184,6 +305,8 @@ kpm_status build_graph(kpm_batch_s* b, const BatchConfig& c) {
     return fail(KPM_EINVAL, "R-tiles must divide the chunks per row");
   if (c.res && c.rtiles > 1)
     return fail(KPM_EINVAL, "the resident form runs untiled instances (R-tiles 1)");
+  if (c.res == FORM_COLS && !cols_kind(b))
+    return fail(KPM_EINVAL, "the column-strip form takes 2D and 3D stencils of uniform real hopping");
   if (c.res && !b->handles[0]->stencil)
     return fail(KPM_EINVAL, "the resident and staged forms take stencil operators only");
   if (c.res == FORM_STAGED && !staged_ok(b))
@@ -191,6 +314,33 @@ kpm_status build_graph(kpm_batch_s* b, const BatchConfig& c) {
   if (b->exec) {
     cudaGraphExecDestroy(b->exec);
     b->exec = nullptr;
+  }
+  ColsPlan cp;
+  if (c.res == FORM_COLS) {
+    if (!plan_cols(b, c.C, &cp))
+      return fail(KPM_EINVAL, "cluster size " + std::to_string(c.C) +
+                                  " cannot be launched with the vectors in column strips");
+    // a replay of an earlier configuration may still be using the old tasks
+    KPM_CUDA(cudaDeviceSynchronize());
+    if (b->ctasks_cap < cp.tasks.size()) {
+      if (b->d_ctasks) cudaFree(b->d_ctasks);
+      b->d_ctasks = nullptr;
+      b->ctasks_cap = 0;
+      KPM_CUDA(cudaMalloc((void**)&b->d_ctasks, cp.tasks.size() * sizeof(ColsTask)));
+      b->ctasks_cap = cp.tasks.size();
+    }
+    if (b->cpart_cap < cp.part) {
+      if (b->d_cpart) cudaFree(b->d_cpart);
+      b->d_cpart = nullptr;
+      b->cpart_cap = 0;
+      KPM_CUDA(cudaMalloc((void**)&b->d_cpart, cp.part * sizeof(double)));
+      b->cpart_cap = cp.part;
+    }
+    for (ColsTask& t : cp.tasks)
+      t.part = c.C > 1 ? (double*)((char*)b->d_cpart + (size_t)t.part) : nullptr;
+    KPM_CUDA(cudaMemcpy(b->d_ctasks, cp.tasks.data(), cp.tasks.size() * sizeof(ColsTask),
+                        cudaMemcpyHostToDevice));
+    b->grid = cp.clusters * c.C;
   }
   // tasks of this configuration: instances in decreasing work, the `top`
   // largest split into rtiles column tiles (consecutive in the queue)
@@ -213,20 +363,24 @@ kpm_status build_graph(kpm_batch_s* b, const BatchConfig& c) {
   // the kernel's shared memory is sized for the widest task
   b->proto = b->host_tasks.back().a;
   const int ntasks = (int)b->host_tasks.size();
-  const int nclu = cfg_clusters(b, c);
+  const int nclu = c.res == FORM_COLS ? cp.clusters : cfg_clusters(b, c);
   if (nclu <= 0)
     return fail(KPM_EINVAL, "cluster size " + std::to_string(c.C) + " cannot be launched" +
                                 (c.res ? " with the vectors resident in shared memory" : ""));
   const int use = std::max(1, std::min(ntasks, nclu * c.frac / 100));
-  b->grid = use * c.C;
+  if (c.res != FORM_COLS) b->grid = use * c.C;
   KPM_CUDA(cudaMemcpy(b->d_tasks, b->host_tasks.data(), b->host_tasks.size() * sizeof(BatchTask),
                       cudaMemcpyHostToDevice));
   const uint64_t before = g_launches.load();
   KPM_CUDA(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = cudaMemsetAsync(b->d_queue, 0, (1 + (size_t)b->count) * sizeof(int), b->cap_stream);
+  cudaError_t e = cudaMemsetAsync(b->d_queue, 0, (1 + 2 * (size_t)b->count) * sizeof(int), b->cap_stream);
   if (e == cudaSuccess)
     e = cudaEventRecordWithFlags(b->ev[0], b->cap_stream, cudaEventRecordExternal);
-  if (e == cudaSuccess && c.res == FORM_STAGED) {
+  if (e == cudaSuccess && c.res == FORM_COLS) {
+    const kpm_handle_s* h0 = b->handles[0];
+    e = launch_cols(b->fp32, h0->geom.dims, h0->has_onsite, b->d_ctasks, (int)cp.tasks.size(),
+                    b->d_queue, cp.clusters, c.C, cp.smem, b->cap_stream);
+  } else if (e == cudaSuccess && c.res == FORM_STAGED) {
     const StgShape sh = stg_shape(b, c.chunk);
     e = b->fp32 ? launch_batch_stg_f32(b->cplx, b->proto, b->d_tasks, ntasks, b->d_queue, b->grid,
                                        c.C, sh.Tl, sh.Sl, sh.SWl, b->cap_stream)
@@ -277,7 +431,7 @@ std::string tune_key(const kpm_batch_s* b) {
   }
   const kpm_handle_s* h = b->handles[0];
   char buf[512];
-  snprintf(buf, sizeof(buf), "batch|%s|fp32=%d|cplx=%d|stencil=%d|dims=%d|hop=%d|ds=%d|ell=%d|R=%d|n=%d|rows=%llu|work=%llu",
+  snprintf(buf, sizeof(buf), "batch|%s|forms=4|fp32=%d|cplx=%d|stencil=%d|dims=%d|hop=%d|ds=%d|ell=%d|R=%d|n=%d|rows=%llu|work=%llu",
            device_name(b->device).c_str(), (int)b->fp32, (int)b->cplx, (int)h->stencil,
            h->geom.dims, (int)h->has_hop, (int)h->has_onsite, h->ell_w, b->R, b->count,
            (unsigned long long)rows, (unsigned long long)work);
@@ -301,8 +455,10 @@ bool cache_lookup(const std::string& key, BatchConfig* c) {
     const size_t sep = s.rfind(" = ");
     if (sep == std::string::npos || s.substr(0, sep) != key) continue;
     BatchConfig t;
-    const int got = sscanf(s.c_str() + sep + 3, "%d %d %d %d %d %d %d", &t.C, &t.chunk, &t.frac,
-                           &t.rtiles, &t.top, &t.res, &t.tpr);
+    int cols = 0;
+    const int got = sscanf(s.c_str() + sep + 3, "%d %d %d %d %d %d %d %d", &t.C, &t.chunk, &t.frac,
+                           &t.rtiles, &t.top, &t.res, &t.tpr, &cols);
+    if (got == 8 && cols == 1) t.res = FORM_COLS;
     if (got == 3) t.rtiles = 1;  // entries written before R-tiling was tuned
     if (got <= 4) t.top = 0;
     if (got <= 5) t.res = 0;     // entries written before the resident form was tuned
@@ -322,9 +478,15 @@ void cache_store(const std::string& key, const BatchConfig& c) {
   if (slash != std::string::npos && slash > 0) mkdir(path.substr(0, slash).c_str(), 0755);
   FILE* f = fopen(path.c_str(), "a");
   if (!f) return;  // an unwritable cache only costs a re-tune
-  fprintf(f, "%s = %d %d %d %d %d %d %d\n", key.c_str(), c.C, c.chunk, c.frac, c.rtiles, c.top,
-          c.res, c.tpr);
+  fprintf(f, "%s = %d %d %d %d %d %d %d %d\n", key.c_str(), c.C, c.chunk, c.frac, c.rtiles, c.top,
+          c.res == FORM_COLS ? 0 : c.res, c.tpr, c.res == FORM_COLS ? 1 : 0);
   fclose(f);
+}
+
+// A call that sets part of another form's configuration goes back to the
+// global-memory form's defaults first.
+void leave_cols(kpm_batch_s* b) {
+  if (b->cfg.res == FORM_COLS) b->cfg = BatchConfig{};
 }
 
 }  // namespace
@@ -422,7 +584,7 @@ kpm_status kpm_batch_create(int count, const kpm_handle* handles, const kpm_para
   e = cudaMalloc(&b->d_pool, std::max<size_t>(off, 256));
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaMalloc(batch pool)"));
   e = cudaMalloc((void**)&b->d_tasks, (size_t)count * MAX_RTILES * sizeof(BatchTask));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_queue, (1 + (size_t)count) * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_queue, (1 + 2 * (size_t)count) * sizeof(int));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreate(&b->ev[0]);
   if (e == cudaSuccess) e = cudaEventCreate(&b->ev[1]);
@@ -503,6 +665,13 @@ kpm_status kpm_batch_create(int count, const kpm_handle* handles, const kpm_para
   });
   b->inst_tasks = tasks;
   b->proto = tasks[b->order[0]].a;
+  // the column strips where they fit: a batch product of the other forms is a
+  // chain of L2 round trips (the 256-instance 2D batch: 38 ms), this one stays
+  // on its SM
+  if (const int C = cols_cluster(b)) {
+    b->cfg.res = FORM_COLS;
+    b->cfg.C = C;
+  }
   BatchConfig cached;
   if (cache_lookup(tune_key(b), &cached)) {
     b->cfg = cached;
@@ -539,6 +708,12 @@ kpm_status kpm_batch_run(kpm_batch b, double* mu, void* stream) {
                         cudaMemcpyDeviceToHost));
     int bad = 0;
     for (auto& t : back) bad |= t.flags;
+    if (b->exec_cfg.res == FORM_COLS) {
+      std::vector<int> fl(b->count);
+      KPM_CUDA(cudaMemcpy(fl.data(), b->d_queue + 1 + b->count, b->count * sizeof(int),
+                          cudaMemcpyDeviceToHost));
+      for (int f : fl) bad |= f;
+    }
     if (bad & BATCH_FLAG_TIMEOUT)
       return fail(KPM_ETIMEOUT, "a bounded wait of the staged batch kernel ran out");
     if (bad)
@@ -579,6 +754,14 @@ kpm_status kpm_batch_tune(kpm_batch b, int reps, void* stream) {
     }
     return KPM_OK;
   };
+  // the column strips at their estimated best cluster size
+  if (const int C = cols_cluster(b)) {
+    BatchConfig c;
+    c.C = C;
+    c.res = FORM_COLS;
+    kpm_status s_ = time_cfg(c);
+    if (s_ != KPM_OK) return s_;
+  }
   // untiled: cluster size, chunk, resident clusters
   for (int C : Cs)
     for (int ch : chunks)
@@ -681,6 +864,7 @@ kpm_status kpm_batch_set_config(kpm_batch b, int cluster, int chunk, int percent
   if (cluster < 1 || cluster > 16 || (cluster & (cluster - 1)) || chunk < 1 || percent < 1 ||
       percent > 100)
     return fail(KPM_EINVAL, "bad batch configuration");
+  leave_cols(b);
   b->cfg.C = cluster;
   b->cfg.chunk = chunk;
   b->cfg.frac = percent;
@@ -692,8 +876,9 @@ kpm_status kpm_batch_set_rtiles(kpm_batch b, int rtiles, int top) {
   if (rtiles < 1 || rtiles > MAX_RTILES || (rtiles & (rtiles - 1)) || (b->G * b->cfg.tpr) % rtiles)
     return fail(KPM_EINVAL, "R-tiles must be 1, 2 or 4 and divide the chunks per row (" +
                                 std::to_string(b->G * b->cfg.tpr) + ")");
-  if (rtiles > 1 && b->cfg.res)
+  if (rtiles > 1 && b->cfg.res && b->cfg.res != FORM_COLS)
     return fail(KPM_EINVAL, "the resident form runs untiled instances (R-tiles 1)");
+  leave_cols(b);
   b->cfg.rtiles = rtiles;
   b->cfg.top = top <= 0 || top >= b->count ? 0 : top;
   return KPM_OK;
@@ -705,10 +890,11 @@ kpm_status kpm_batch_set_chunk_bytes(kpm_batch b, int bytes) {
   const int tpr = bytes == 16 ? 2 : 1;
   if (tpr == 2 && !half_chunks_ok(b))
     return fail(KPM_EINVAL, "16-byte chunks take real FP32 vectors and stencil operators");
-  if (tpr == 2 && b->cfg.res)
+  if (tpr == 2 && b->cfg.res && b->cfg.res != FORM_COLS)
     return fail(KPM_EINVAL, "the resident form runs 32-byte chunks");
   if ((b->G * tpr) % b->cfg.rtiles)
     return fail(KPM_EINVAL, "the current R-tiles do not divide the chunks per row");
+  leave_cols(b);
   b->cfg.tpr = tpr;
   return KPM_OK;
 }
@@ -727,6 +913,7 @@ kpm_status kpm_batch_set_resident(kpm_batch b, int resident) {
     return fail(KPM_EINVAL, "the resident form takes stencil operators only");
   if (resident && b->cfg.tpr != 1)
     return fail(KPM_EINVAL, "the resident form runs 32-byte chunks");
+  leave_cols(b);
   b->cfg.res = resident ? FORM_RESIDENT : FORM_GLOBAL;
   if (resident) {
     b->cfg.rtiles = 1;
@@ -758,6 +945,7 @@ kpm_status kpm_batch_set_staged(kpm_batch b, int staged) {
     return fail(KPM_EINVAL, "the staged form takes stencil operators with rows of at most 32 chunks");
   if (staged && b->cfg.tpr != 1)
     return fail(KPM_EINVAL, "the staged form runs 32-byte chunks");
+  leave_cols(b);
   if (staged) {
     b->cfg.res = FORM_STAGED;
     b->cfg.rtiles = 1;
@@ -777,6 +965,30 @@ kpm_status kpm_batch_get_staged(kpm_batch b, int* staged, int* tile_rows, int* s
   return KPM_OK;
 }
 
+kpm_status kpm_batch_set_columns(kpm_batch b, int columns) {
+  if (!b) return fail(KPM_EINVAL, "batch is NULL");
+  if (columns != 0 && columns != 1) return fail(KPM_EINVAL, "columns must be 0 or 1");
+  if (!columns) {
+    leave_cols(b);
+    return KPM_OK;
+  }
+  KPM_CUDA(cudaSetDevice(b->device));
+  const int C = cols_cluster(b);
+  if (!C)
+    return fail(KPM_EINVAL,
+                "the column strips take 2D and 3D stencils of uniform real hopping that fit a cluster");
+  b->cfg = BatchConfig{};
+  b->cfg.res = FORM_COLS;
+  b->cfg.C = C;
+  return KPM_OK;
+}
+
+kpm_status kpm_batch_get_columns(kpm_batch b, int* columns) {
+  if (!b) return fail(KPM_EINVAL, "batch is NULL");
+  if (columns) *columns = b->cfg.res == FORM_COLS;
+  return KPM_OK;
+}
+
 kpm_status kpm_batch_get_rtiles(kpm_batch b, int* rtiles, int* top, int* max_rtiles) {
   if (!b) return fail(KPM_EINVAL, "batch is NULL");
   if (rtiles) *rtiles = b->cfg.rtiles;
@@ -793,6 +1005,8 @@ void kpm_batch_destroy(kpm_batch b) {
   if (b->d_pool) cudaFree(b->d_pool);
   if (b->d_tasks) cudaFree(b->d_tasks);
   if (b->d_queue) cudaFree(b->d_queue);
+  if (b->d_ctasks) cudaFree(b->d_ctasks);
+  if (b->d_cpart) cudaFree(b->d_cpart);
   if (b->ev[0]) cudaEventDestroy(b->ev[0]);
   if (b->ev[1]) cudaEventDestroy(b->ev[1]);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);

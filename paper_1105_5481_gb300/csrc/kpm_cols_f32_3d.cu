@@ -1,0 +1,17 @@
+// Column-strip solve: FP32 vectors, 3D stencils.
+#include "kpm_cols.cuh"
+
+namespace kpm {
+
+cudaError_t launch_cols_f32_3d(bool ds, const ColsTask* tasks, int ntasks, int* queue, int clusters,
+                                int C, size_t smem, cudaStream_t st) {
+  return ds ? cols::launch<float, 3, true>(tasks, ntasks, queue, clusters, C, smem, st)
+            : cols::launch<float, 3, false>(tasks, ntasks, queue, clusters, C, smem, st);
+}
+
+int cols_clusters_f32_3d(bool ds, int C, size_t smem) {
+  return ds ? cols::max_clusters<float, 3, true>(C, smem)
+            : cols::max_clusters<float, 3, false>(C, smem);
+}
+
+}  // namespace kpm

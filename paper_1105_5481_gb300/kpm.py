@@ -112,6 +112,8 @@ def lib() -> C.CDLL:
         L.kpm_batch_set_staged.argtypes = [h, C.c_int]
         L.kpm_batch_get_staged.argtypes = [h, C.POINTER(C.c_int), C.POINTER(C.c_int),
                                            C.POINTER(C.c_int)]
+        L.kpm_batch_set_columns.argtypes = [h, C.c_int]
+        L.kpm_batch_get_columns.argtypes = [h, C.POINTER(C.c_int)]
         L.kpm_batch_destroy.argtypes = [h]
         L.kpm_batch_destroy.restype = None
         L.kpm_server_create.argtypes = [C.c_size_t, C.c_int, C.c_int, C.POINTER(h)]
@@ -571,6 +573,18 @@ def kpm_batch_get_staged(bt: Batch):
     on, tr, st = C.c_int(), C.c_int(), C.c_int()
     _check(lib().kpm_batch_get_staged(bt.raw, C.byref(on), C.byref(tr), C.byref(st)))
     return bool(on.value), tr.value, st.value
+
+
+def kpm_batch_set_columns(bt: Batch, columns=True):
+    """Run the vector columns as independent tasks held on the SMs."""
+    _check(lib().kpm_batch_set_columns(bt.raw, int(bool(columns))))
+
+
+def kpm_batch_get_columns(bt: Batch):
+    """Whether the column-strip form is set."""
+    on = C.c_int()
+    _check(lib().kpm_batch_get_columns(bt.raw, C.byref(on)))
+    return bool(on.value)
 
 
 def kpm_batch_info(bt: Batch):
