@@ -181,12 +181,17 @@ bool setup_dense_tc(kpm_handle_s* h, int Rp) {
   auto* d = new DenseTC;
   d->n = h->n;
   d->Rp = Rp;
+  d->crt = h->n <= DENSE_TC_CRT_MAX_N;
+  d->nq = d->crt ? (int)((h->n + 7) / 8 * 8) : 0;
+  d->Rq = (Rp + 7) / 8 * 8;
   dense_tc_split(h->n, &d->beta, &d->k);
-  const size_t n = (size_t)h->n, k = (size_t)d->k;
-  const size_t cbytes = dense_tc_c_floats(h->n, Rp, d->k) * sizeof(float);
+  const size_t n = (size_t)h->n, k = d->crt ? DENSE_TC_MODULI : (size_t)d->k;
+  const size_t na = d->crt ? n * d->nq : n * n, nb = d->crt ? (size_t)d->nq * d->Rq : n * Rp;
+  const size_t cbytes =
+      (d->crt ? k * n * d->Rq : dense_tc_c_floats(h->n, Rp, d->k)) * sizeof(float);
   d->ws_bytes = 32u << 20;
   bool ok = cbytes <= ((size_t)64 << 30) && dalloc((char**)&d->workspace, d->ws_bytes) == KPM_OK &&
-            dalloc(&d->A, k * n * n) == KPM_OK && dalloc(&d->B, k * n * Rp) == KPM_OK &&
+            dalloc(&d->A, k * na) == KPM_OK && dalloc(&d->B, k * nb) == KPM_OK &&
             dalloc((char**)&d->C, cbytes) == KPM_OK && dalloc(&d->row_scale, n) == KPM_OK &&
             dalloc(&d->col_scale, (size_t)Rp) == KPM_OK && dalloc(&d->cmax, (size_t)Rp) == KPM_OK;
   w.dtc = d;

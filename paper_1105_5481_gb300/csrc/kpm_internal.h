@@ -62,8 +62,14 @@ struct ColresPlan {
 // Dense products on the bf16 tensor cores by the Ozaki splitting scheme
 // (kpm_dense_tc.cu), real FP64 dense handles: slices of S (per call) and of
 // the current vector block (per step), the exact slice products, exponents.
+constexpr int DENSE_TC_MODULI = 19;
+constexpr int64_t DENSE_TC_CRT_MAX_N = 4096;
 struct DenseTC {
   int64_t n = 0;
+  // the residue form (n <= DENSE_TC_CRT_MAX_N): A bf16 [19][n][nq], B bf16
+  // [19][nq][Rq], C [19][n][Rq], n and Rp rounded up to 8
+  bool crt = false;
+  int nq = 0, Rq = 0;
   int Rp = 0, beta = 0, k = 0;
   void* blas = nullptr;             // cublasHandle_t
   void* workspace = nullptr;        // the cuBLAS workspace (no allocation during capture)
