@@ -1677,14 +1677,16 @@ kpm_status kpm_thermo(const double* mu, int M, double a, double b, int K, int ke
   if (s_ != KPM_OK) return s_;
   cudaStream_t st = (cudaStream_t)stream;
   const bool dmu = is_device_ptr(mu), dout = is_device_ptr(out);
-  // work: coef[M] table[4K] E[K] rho[K] (+ mu[M] beta[nT] out[4 nT] staging)
-  const size_t nwork = (size_t)M + 6 * (size_t)K + (dmu ? 0 : M) + (dbeta ? 0 : nT) +
+  // work: coef[M] table[4K] E[K] rho[K] part (+ mu[M] beta[nT] out[4 nT] staging)
+  const size_t npart = thermo_part_doubles(K, nT);
+  const size_t nwork = (size_t)M + 6 * (size_t)K + npart + (dmu ? 0 : M) + (dbeta ? 0 : nT) +
                        (dout ? 0 : 4 * (size_t)nT);
   double* work = nullptr;
   KPM_CUDA(cudaMallocAsync((void**)&work, nwork * sizeof(double), st));
   double* E_d = work + M + 4 * (size_t)K;
   double* rho_d = E_d + K;
-  double* cur = rho_d + K;
+  double* part = rho_d + K;
+  double* cur = part + npart;
   const double* mu_d = mu;
   const double* beta_d = beta;
   double* out_d = out;
@@ -1701,7 +1703,7 @@ kpm_status kpm_thermo(const double* mu, int M, double a, double b, int K, int ke
   }
   if (!dout) { out_d = cur; cur += 4 * (size_t)nT; }
   if (e == cudaSuccess) e = launch_dos(mu_d, M, a, b, K, kernel, lambda, E_d, rho_d, work, st);
-  if (e == cudaSuccess) e = launch_thermo(E_d, rho_d, K, a, beta_d, nT, mu_c, out_d, st);
+  if (e == cudaSuccess) e = launch_thermo(E_d, rho_d, K, a, beta_d, nT, mu_c, work + M, part, out_d, st);
   if (e == cudaSuccess && !dout)
     e = cudaMemcpyAsync(out, out_d, 4 * (size_t)nT * sizeof(double), cudaMemcpyDeviceToHost, st);
   cudaFreeAsync(work, st);
@@ -1723,10 +1725,11 @@ static kpm_status stats_to(const double* pv_d, int nvec, int M, double a, double
     host[i] = outs[i] && !is_device_ptr(outs[i]);
     if (host[i]) stage += len[i];
   }
-  const size_t nwork = (size_t)M + 4 * (size_t)K + (size_t)K * nvec + stage;
+  const size_t nstat = stats_work_doubles(nvec, M, K);
+  const size_t nwork = nstat + stage;
   double* work = nullptr;
   KPM_CUDA(cudaMallocAsync((void**)&work, nwork * sizeof(double), st));
-  double* cur = work + M + 4 * (size_t)K + (size_t)K * nvec;
+  double* cur = work + nstat;
   double* dst[5];
   for (int i = 0; i < 5; ++i) {
     dst[i] = outs[i];

@@ -854,23 +854,28 @@ __global__ void green_kernel(const double* __restrict__ coef, int M, double a, d
   }
 }
 
-// Fermi-occupation integrals of the DOS on the K nodes, one CTA per inverse
-// temperature beta[t] (Gauss-Chebyshev weights w_k = a pi sin(theta_k) / K):
-// out[t] = (n, u, s, c) per site with f = 1/(1 + e^x), x = beta (E - mu_c):
+// Fermi-occupation integrals of the DOS on the K nodes (Gauss-Chebyshev weights
+// w_k = a pi sin(theta_k) / K, the sine from the DOS's table): the CTA
+// (blockIdx.x, t) adds its share of the nodes for the inverse temperature
+// beta[t] into part[t][blockIdx.x][4].  About 100 FP64 instructions per node
+// and temperature (exp, log1p, a division) at 2 per SM and clock: one CTA per
+// temperature left most of the SMs idle.
+// The sums are (n, u, s, c) per site with f = 1/(1 + e^x), x = beta (E - mu_c):
 //   n = sum w rho f,  u = sum w rho E f,
 //   s = sum w rho [min(f, 1-f) |x| + log1p(e^-|x|)],  c = sum w rho x^2 f (1-f);
 // beta = +inf is the ground state (f = step, s = c = 0).
 __global__ void __launch_bounds__(LZ_BLOCK) thermo_kernel(const double* __restrict__ E,
                                                           const double* __restrict__ rho, int K,
                                                           double a, const double* __restrict__ beta,
-                                                          double mu_c, double* out) {
+                                                          double mu_c,
+                                                          const double* __restrict__ table,
+                                                          double* part) {
   __shared__ double red[LZ_WARPS * 4];
-  const double bt = beta[blockIdx.x];
+  const double bt = beta[blockIdx.y], w0 = a * M_PI / (double)K;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int k = threadIdx.x; k < K; k += LZ_BLOCK) {
-    double sx, cx;
-    sincospi(((double)k + 0.5) / (double)K, &sx, &cx);
-    const double wr = a * M_PI * sx / (double)K * rho[k];
+  for (int k = blockIdx.x * LZ_BLOCK + threadIdx.x; k < K; k += gridDim.x * LZ_BLOCK) {
+    const double sx = table[(2LL * k + 1 + 3LL * K) % (4LL * K)];
+    const double wr = w0 * sx * rho[k];
     const double e = E[k], d = e - mu_c;
     double f, ent = 0.0, cv = 0.0;
     if (isinf(bt)) {
@@ -888,7 +893,17 @@ __global__ void __launch_bounds__(LZ_BLOCK) thermo_kernel(const double* __restri
     acc[3] = fma(wr, cv, acc[3]);
   }
   const double tot = block_multi_sum<4>(acc, red);
-  if (threadIdx.x < 4) out[(size_t)blockIdx.x * 4 + threadIdx.x] = tot;
+  if (threadIdx.x < 4)
+    part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 4 + threadIdx.x] = tot;
+}
+
+// out[t][q] = the CTAs' shares in their order
+__global__ void thermo_sum_kernel(const double* __restrict__ part, int nblk, int nT, double* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= 4 * nT) return;
+  double s = 0.0;
+  for (int b = 0; b < nblk; ++b) s += part[((size_t)(i >> 2) * nblk + b) * 4 + (i & 3)];
+  out[i] = s;
 }
 
 // Mean and standard error over nvec vectors of each moment: pv[r * M + n].
@@ -908,22 +923,101 @@ __global__ void moment_stats_kernel(const double* __restrict__ pv, int nvec, int
   }
 }
 
-// One CTA (LZ_BLOCK threads) per node k: the DOS of every vector's moments
-// (Eq. (fKPM) with the damping in g, which carries the factor 2 of n >= 1),
-// eight vectors at a time, kept in scratch[k * nvec + r]; then their mean and
-// standard error (two passes).
-__global__ void __launch_bounds__(LZ_BLOCK) dos_stats_kernel(
-    const double* __restrict__ pv, const double* __restrict__ g, int nvec, int M, double a,
-    double b, int K, const double* __restrict__ table, double* scratch, double* E, double* rmean,
-    double* rerr) {
+// The DOS of every vector (Eq. (fKPM); g carries the damping and the factor 2
+// of n >= 1) by one Cooley-Tukey step where K has a divisor N1 near sqrt(M):
+// with n = n1 + N1 n2, theta_k = pi (2k+1) / (2K) and K' = K / N1,
+//   sum_n c_n cos(n theta_k) = Re sum_n1 e^{i n1 theta_k} D[n1][k'],
+//   D[n1][k'] = sum_n2 c_{n1 + N1 n2} e^{i pi n2 (2k'+1) / (2K')},
+// because e^{i N1 n2 theta_k} depends on 2k+1 mod 4K' alone (the upper half of
+// the residues conjugate to the lower), so that D has K entries per vector.
+// 2 M / N1 + 2 N1 FMAs per node and vector instead of M: on GB300's FP64 pipe
+// (2 per SM and clock) the direct sum for 64 vectors of 2048 moments on 4096
+// nodes is 0.85 ms of FMAs alone; kpm_stats and 16 temperatures of kpm_thermo
+// on these sizes take 0.81 ms in all with this split and the integrals spread
+// over the chip, 2.12 ms before.  Every angle is a whole multiple of pi / (2K), its
+// cosine and sine read from the table at the reduced index.
+//
+// Stage 1: one thread per (n1, k'), eight vectors: D as (re, im) [r][n1][k'].
+constexpr int DOS_VECS = 8;
+__global__ void __launch_bounds__(128) dos_inner_kernel(const double* __restrict__ pv,
+                                                        const double* __restrict__ g, int nvec, int M,
+                                                        int K, int N1,
+                                                        const double* __restrict__ table,
+                                                        double2* __restrict__ D) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= K) return;
+  const int Kp = K / N1, n1 = e / Kp, kp = e - n1 * Kp, r0 = blockIdx.y * DOS_VECS;
+  const int64_t n4 = 4LL * K, step = (2LL * kp + 1) * N1;  // in units of pi / (2K); step < 2K
+  const double* p[DOS_VECS];
+#pragma unroll
+  for (int i = 0; i < DOS_VECS; ++i) p[i] = pv + (size_t)min(r0 + i, nvec - 1) * M;
+  double re[DOS_VECS], im[DOS_VECS];
+#pragma unroll
+  for (int i = 0; i < DOS_VECS; ++i) re[i] = im[i] = 0.0;
+  int64_t j = 0;
+  for (int n = n1; n < M; n += N1) {
+    const int64_t js = j >= K ? j - K : j + 3LL * K;
+    const double c = g[n] * table[j], s = g[n] * table[js];
+#pragma unroll
+    for (int i = 0; i < DOS_VECS; ++i) {
+      const double v = p[i][n];
+      re[i] = fma(v, c, re[i]);
+      im[i] = fma(v, s, im[i]);
+    }
+    j += step;
+    if (j >= n4) j -= n4;
+  }
+#pragma unroll
+  for (int i = 0; i < DOS_VECS; ++i)
+    if (r0 + i < nvec) D[(size_t)(r0 + i) * K + e] = make_double2(re[i], im[i]);
+}
+
+// Stage 2: one thread per node, eight vectors; scratch[r][k] = the DOS.
+__global__ void __launch_bounds__(128) dos_outer_kernel(const double2* __restrict__ D, int nvec, double a,
+                                                        int K, int N1,
+                                                        const double* __restrict__ table,
+                                                        double* __restrict__ scratch) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= K) return;
+  const int Kp = K / N1, r0 = blockIdx.y * DOS_VECS;
+  const int64_t n4 = 4LL * K, step = 2LL * k + 1;
+  const int64_t res = step % (4LL * Kp);
+  const bool conj = res > 2LL * Kp;
+  const int kp = (int)((conj ? 4LL * Kp - res : res) / 2);
+  const double2* d[DOS_VECS];
+#pragma unroll
+  for (int i = 0; i < DOS_VECS; ++i) d[i] = D + (size_t)min(r0 + i, nvec - 1) * K + kp;
+  double acc[DOS_VECS];
+#pragma unroll
+  for (int i = 0; i < DOS_VECS; ++i) acc[i] = 0.0;
+  int64_t j = 0;
+  for (int n1 = 0; n1 < N1; ++n1) {
+    const int64_t js = j >= K ? j - K : j + 3LL * K;
+    const double c = table[j], s = conj ? table[js] : -table[js];
+#pragma unroll
+    for (int i = 0; i < DOS_VECS; ++i) {
+      const double2 v = d[i][(size_t)n1 * Kp];
+      acc[i] = fma(c, v.x, acc[i]);
+      acc[i] = fma(s, v.y, acc[i]);
+    }
+    j += step;
+    if (j >= n4) j -= n4;
+  }
+  const double scale = 1.0 / (M_PI * table[(step + 3LL * K) % n4]) / a;
+#pragma unroll
+  for (int i = 0; i < DOS_VECS; ++i)
+    if (r0 + i < nvec) scratch[(size_t)(r0 + i) * K + k] = acc[i] * scale;
+}
+
+// Where K has no such divisor: the direct sums, one CTA (LZ_BLOCK threads) per
+// node, eight vectors at a time, into scratch[r][k].
+__global__ void __launch_bounds__(LZ_BLOCK) dos_direct_kernel(
+    const double* __restrict__ pv, const double* __restrict__ g, int nvec, int M, double a, int K,
+    const double* __restrict__ table, double* scratch) {
   __shared__ double red[LZ_WARPS * 8];
-  __shared__ double s_mean;
   const int k = blockIdx.x;
   const int64_t step = 2LL * k + 1, n4 = 4LL * K;
-  double sx, cx;
-  sincospi(((double)k + 0.5) / (double)K, &sx, &cx);
-  const double scale = 1.0 / (M_PI * sx) / a;
-  double* rk = scratch + (size_t)k * nvec;
+  const double scale = 1.0 / (M_PI * table[(step + 3LL * K) % n4]) / a;
   for (int r0 = 0; r0 < nvec; r0 += 8) {
     double acc[8];
 #pragma unroll
@@ -935,27 +1029,58 @@ __global__ void __launch_bounds__(LZ_BLOCK) dos_stats_kernel(
         if (r0 + i < nvec) acc[i] = fma(pv[(size_t)(r0 + i) * M + n], t, acc[i]);
     }
     const double tot = block_multi_sum<8>(acc, red);
-    if ((int)threadIdx.x < 8 && r0 + (int)threadIdx.x < nvec) rk[r0 + threadIdx.x] = tot * scale;
+    if ((int)threadIdx.x < 8 && r0 + (int)threadIdx.x < nvec)
+      scratch[(size_t)(r0 + threadIdx.x) * K + k] = tot * scale;
     __syncthreads();
   }
-  double v[1] = {0.0};
-  for (int r = threadIdx.x; r < nvec; r += LZ_BLOCK) v[0] += rk[r];
-  double tot = block_multi_sum<1>(v, red);
-  if (threadIdx.x == 0) s_mean = tot / nvec;
-  __syncthreads();
-  const double m = s_mean;
-  v[0] = 0.0;
-  for (int r = threadIdx.x; r < nvec; r += LZ_BLOCK) {
-    const double d = rk[r] - m;
-    v[0] = fma(d, d, v[0]);
+}
+
+// Mean and standard error over the vectors of the DOS on each node (two passes).
+__global__ void dos_stats_kernel(const double* __restrict__ scratch, int nvec, double a, double b,
+                                 int K, const double* __restrict__ table, double* E, double* rmean,
+                                 double* rerr) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= K) return;
+  const double* rk = scratch + k;
+  double s = 0.0;
+#pragma unroll 8
+  for (int r = 0; r < nvec; ++r) s += rk[(size_t)r * K];
+  const double m = s / nvec;
+  double v = 0.0;
+  if (rerr) {
+#pragma unroll 8
+    for (int r = 0; r < nvec; ++r) {
+      const double d = rk[(size_t)r * K] - m;
+      v = fma(d, d, v);
+    }
   }
-  __syncthreads();
-  tot = block_multi_sum<1>(v, red);
-  if (threadIdx.x == 0) {
-    if (E) E[k] = a * cx + b;
-    if (rmean) rmean[k] = m;
-    if (rerr) rerr[k] = nvec > 1 ? sqrt(tot / ((double)(nvec - 1) * nvec)) : 0.0;
+  if (E) E[k] = a * table[2LL * k + 1] + b;
+  if (rmean) rmean[k] = m;
+  if (rerr) rerr[k] = nvec > 1 ? sqrt(v / ((double)(nvec - 1) * nvec)) : 0.0;
+}
+
+// The divisor N1 of K of least 2 ceil(M / N1) + 2 N1, or 0 where that is not
+// well below the M FMAs of the direct sum (K prime, M small).
+static int dos_split(int K, int M) {
+  int best = 0;
+  int64_t cost = (int64_t)M * 6 / 10;
+  for (int d = 2; d <= K && d <= M; ++d) {
+    if (K % d) continue;
+    const int64_t c = 2 * (((int64_t)M + d - 1) / d) + 2LL * d;
+    if (c < cost) {
+      cost = c;
+      best = d;
+    }
+    if (2LL * d > cost) break;
   }
+  return best;
+}
+
+// Vectors per pass of the split DOS: D (two doubles per vector and node)
+// within 64 MB, at least eight.
+static int dos_pass(int nvec, int K) {
+  const int64_t fit = ((int64_t)4 << 20) / K / DOS_VECS * DOS_VECS;
+  return (int)std::min<int64_t>(std::min<int64_t>(nvec, std::max<int64_t>(DOS_VECS, fit)), 32768 * DOS_VECS);
 }
 
 }  // namespace
@@ -1169,12 +1294,12 @@ cudaError_t launch_tridiag_bounds(const double* alpha, const double* beta, int m
 cudaError_t launch_stats(const double* pv, int nvec, int M, double a, double b, int K, int kernel,
                          double lambda, double* mu_mean, double* mu_err, double* E, double* rmean,
                          double* rerr, double* work, cudaStream_t st) {
-  // work: g[M], table[4K], scratch[K * nvec]
+  // work: stats_work_doubles() doubles
   double* g = work;
-  double* table = work + M;
+  double* table = work + ((size_t)M + 1) / 2 * 2;
   double* scratch = table + 4 * (size_t)K;
   if (mu_mean || mu_err) {
-    moment_stats_kernel<<<blocks_for(M, 256), 256, 0, st>>>(pv, nvec, M, mu_mean, mu_err);
+    moment_stats_kernel<<<blocks_for(M, FP64_SPREAD), FP64_SPREAD, 0, st>>>(pv, nvec, M, mu_mean, mu_err);
     counted(cudaSuccess);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1188,9 +1313,34 @@ cudaError_t launch_stats(const double* pv, int nvec, int M, double a, double b, 
   counted(cudaSuccess);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  dos_stats_kernel<<<K, LZ_BLOCK, 0, st>>>(pv, g, nvec, M, a, b, K, table, scratch, E, rmean,
-                                           rerr);
+  if (rmean || rerr) {
+    if (const int N1 = dos_split(K, M)) {
+      double2* D = reinterpret_cast<double2*>(scratch + ((size_t)K * nvec + 1) / 2 * 2);
+      const int pass = dos_pass(nvec, K);
+      for (int r0 = 0; r0 < nvec; r0 += pass) {
+        const int nr = std::min(pass, nvec - r0);
+        const dim3 grid((unsigned)((K + 127) / 128), (unsigned)((nr + DOS_VECS - 1) / DOS_VECS));
+        dos_inner_kernel<<<grid, 128, 0, st>>>(pv + (size_t)r0 * M, g, nr, M, K, N1, table, D);
+        counted(cudaSuccess);
+        dos_outer_kernel<<<grid, 128, 0, st>>>(D, nr, a, K, N1, table, scratch + (size_t)r0 * K);
+        counted(cudaSuccess);
+      }
+    } else {
+      dos_direct_kernel<<<K, LZ_BLOCK, 0, st>>>(pv, g, nvec, M, a, K, table, scratch);
+      counted(cudaSuccess);
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  dos_stats_kernel<<<blocks_for(K, FP64_SPREAD), FP64_SPREAD, 0, st>>>(scratch, nvec, a, b, K, table, E,
+                                                                      rmean, rerr);
   return counted(cudaGetLastError());
+}
+
+size_t stats_work_doubles(int nvec, int M, int K) {
+  // g[M], table[4K], scratch[nvec][K] and, 16-byte aligned, D
+  return ((size_t)M + 1) / 2 * 2 + 4 * (size_t)K + ((size_t)K * nvec + 1) / 2 * 2 +
+         (dos_split(K, M) ? 2 * (size_t)dos_pass(nvec, K) * K : 0);
 }
 
 cudaError_t launch_green(const double* mu, int M, double a, double b, int K, int kernel,
@@ -1210,9 +1360,20 @@ cudaError_t launch_green(const double* mu, int M, double a, double b, int K, int
   return counted(cudaGetLastError());
 }
 
+// CTAs per temperature: about two per SM over all temperatures.
+static int thermo_blocks(int K, int nT) {
+  return std::max(1, std::min((K + LZ_BLOCK - 1) / LZ_BLOCK, 304 / std::max(1, nT)));
+}
+
+size_t thermo_part_doubles(int K, int nT) { return (size_t)4 * nT * thermo_blocks(K, nT); }
+
 cudaError_t launch_thermo(const double* E, const double* rho, int K, double a,
-                          const double* beta, int nT, double mu_c, double* out, cudaStream_t st) {
-  thermo_kernel<<<nT, LZ_BLOCK, 0, st>>>(E, rho, K, a, beta, mu_c, out);
+                          const double* beta, int nT, double mu_c, const double* table,
+                          double* part, double* out, cudaStream_t st) {
+  const int nb = thermo_blocks(K, nT);
+  thermo_kernel<<<dim3(nb, nT), LZ_BLOCK, 0, st>>>(E, rho, K, a, beta, mu_c, table, part);
+  counted(cudaSuccess);
+  thermo_sum_kernel<<<blocks_for(4LL * nT, 128), 128, 0, st>>>(part, nb, nT, out);
   return counted(cudaGetLastError());
 }
 

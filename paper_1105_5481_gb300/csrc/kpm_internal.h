@@ -160,14 +160,19 @@ cudaError_t launch_tridiag_bounds(const double* alpha, const double* beta, int m
 cudaError_t launch_dos(const double* mu, int M, double a, double b, int K, int kernel,
                        double lambda, double* E, double* rho, double* work, cudaStream_t st);
 // Fermi-occupation integrals (n, u, s, c per site) of a DOS on the K nodes
+// (table: the cosine table launch_dos left at work + M; part: scratch of
+// thermo_part_doubles)
+size_t thermo_part_doubles(int K, int nT);
 cudaError_t launch_thermo(const double* E, const double* rho, int K, double a,
-                          const double* beta, int nT, double mu_c, double* out, cudaStream_t st);
+                          const double* beta, int nT, double mu_c, const double* table,
+                          double* part, double* out, cudaStream_t st);
 // local Green's function on the K nodes (work holds M + 4K doubles)
 cudaError_t launch_green(const double* mu, int M, double a, double b, int K, int kernel,
                          double lambda, double* E, double* g_re, double* g_im, double* work,
                          cudaStream_t st);
 // mean and standard error over nvec vectors (pv[r*M + n]) of the moments and
-// of the per-vector DOS; any output may be NULL; work holds M + 4K + K*nvec doubles
+// of the per-vector DOS; any output may be NULL; work holds stats_work_doubles
+size_t stats_work_doubles(int nvec, int M, int K);
 cudaError_t launch_stats(const double* pv, int nvec, int M, double a, double b, int K, int kernel,
                          double lambda, double* mu_mean, double* mu_err, double* E, double* rmean,
                          double* rerr, double* work, cudaStream_t st);
