@@ -620,7 +620,8 @@ kpm_status kpm_testing_stall_step_pipeline(int on);
  * step, 2 the dense product on the FP64 pipe, 3 the dense product on the
  * tensor cores, 4 the TMA-fed stencil step, 5 the column-resident solve
  * (all products of a realisation of a small stencil or padded-ELL operator in
- * one cluster launch).  KPM_ENOTREADY before the first kpm_moments call. */
+ * one cluster launch), 6 the column strips (the columns of all S > 1
+ * realisations as tasks of one persistent launch).  KPM_ENOTREADY before the first kpm_moments call. */
 kpm_status kpm_testing_last_step_form(kpm_handle h, int* form);
 
 #ifdef __cplusplus

@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "kpm_colres.h"
+#include "kpm_cols.h"
 #include "kpm_internal.h"
 
 namespace kpm {
@@ -203,6 +204,16 @@ bool setup_dense_tc(kpm_handle_s* h, int Rp) {
   return ok;
 }
 
+void free_cols(kpm_handle_s::Work& w) {
+  dfree(w.cs_tasks);
+  dfree(w.cs_queue);
+  dfree(w.cs_part);
+  w.cs_tasks = nullptr;
+  w.cs_queue = nullptr;
+  w.cs_part = nullptr;
+  w.cs = {};
+}
+
 void free_work(kpm_handle_s* h) {
   auto& w = h->work;
   if (w.exec) cudaGraphExecDestroy(w.exec);
@@ -215,6 +226,7 @@ void free_work(kpm_handle_s* h) {
   dfree(w.v0stage);
   dfree(w.sb_dev);
   dfree(w.cr_gp);
+  free_cols(w);
   if (w.ev[0]) cudaEventDestroy(w.ev[0]);
   if (w.ev[1]) cudaEventDestroy(w.ev[1]);
   w = kpm_handle_s::Work{};
@@ -656,6 +668,7 @@ kpm_status kpm_testing_last_step_form(kpm_handle h, int* form) {
   const auto& w = h->work;
   if (w.M == 0) return fail(KPM_ENOTREADY, "no kpm_moments call has planned its launches yet");
   if (h->dense) *form = w.dtc ? 3 : 2;
+  else if (w.cs.clusters > 0) *form = 6;
   else if (w.cr.C > 0) *form = 5;
   else *form = w.proto.tma_stages > 0 ? (h->stencil ? 4 : 1) : 0;
   return KPM_OK;
@@ -879,7 +892,7 @@ kpm_status kpm_step_timing(kpm_handle h, double* ms, int* step_launches) {
   KPM_CUDA(cudaSetDevice(h->device));
   float t = 0.f;
   KPM_CUDA(cudaEventElapsedTime(&t, h->work.ev[0], h->work.ev[1]));
-  if (ms) *ms = t;
+  if (ms) *ms = h->work.cs.clusters > 0 ? t / h->work.cs.S : t;  // one launch for all realisations
   if (step_launches) *step_launches = h->work.M / 2;
   return KPM_OK;
 }
@@ -1020,6 +1033,97 @@ ColresArgs colres_args(const kpm_handle_s* h, int R, int n0, int n1, int steps, 
   return c;
 }
 
+// Several realisations of a 2D or 3D stencil of uniform real hopping with FP64
+// vectors: their S R columns are independent recursions, so all of them go as
+// column tasks into one persistent launch (kpm_cols.h) when that is estimated
+// faster than S solves one after the other.  A single small realisation leaves
+// most of the FP64 pipes idle (10^3 cube, 14 vectors, 128 realisations, M =
+// 256: 17.7 ms one after the other, 4.9 ms in one launch, 4.2 of it FP64 work).  FP32 vectors keep the
+// solves in turn: their compensated dots depend on the form's sum order.
+bool cols_solve_kind(const kpm_handle_s* h, bool fp32) {
+  return !fp32 && h->stencil && !h->cplx && !h->has_hop && (h->geom.dims == 2 || h->geom.dims == 3);
+}
+
+// Plans the launch for the current buffers; leaves w.cs.clusters 0 where the
+// form does not apply.
+kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps) {
+  auto& w = h->work;
+  free_cols(w);
+  if (S < 2 || !cols_solve_kind(h, false) || getenv("KPM_COLRES")) return KPM_OK;
+  const int dims = h->geom.dims;
+  const bool ds = h->has_onsite;
+  struct Try {
+    ColsShape s;
+    int width, clusters;
+    size_t smem;
+    double us;
+  } best{};
+  best.us = 0.85 * S * (w.cr.C > 0 ? w.cr.us : step_chain_us(h->n, R, false, false, false));
+  for (int C : {1, 2, 4, 8, 16}) {
+    Try t{};
+    if (!cols_shape(h->geom, h->n, R, false, C, &t.s)) continue;
+    t.width = std::min(R, t.s.max_cols);
+    // narrower tasks where the widest leave clusters without work
+    for (;;) {
+      t.smem = cols_smem(t.s, false, t.width);
+      t.clusters = cols_max_clusters(false, dims, ds, C, t.smem);
+      const int64_t tasks = (int64_t)S * ((R + t.width - 1) / t.width);
+      if (t.width == 1 || tasks >= 2 * (int64_t)std::max(1, t.clusters)) break;
+      t.width = (t.width + 1) / 2;
+    }
+    if (t.clusters < 1) continue;
+    const int64_t tasks = (int64_t)S * ((R + t.width - 1) / t.width);
+    t.us = (double)((tasks + t.clusters - 1) / t.clusters) * (t.s.us_fixed + t.width * t.s.us_col);
+    if (t.us < best.us) best = t;
+  }
+  if (best.s.C == 0) return KPM_OK;
+  const int C = best.s.C, groups = (R + best.width - 1) / best.width, ntasks = S * groups;
+  std::vector<ColsTask> tasks;
+  tasks.reserve(ntasks);
+  size_t part = 0;
+  const StepArgs& a = w.proto;
+  for (int s = 0; s < S; ++s)
+    for (int g = 0; g < groups; ++g) {
+      ColsTask t{};
+      const int c0 = (int)((int64_t)R * g / groups), c1 = (int)((int64_t)R * (g + 1) / groups);
+      cols_set_layout(t, best.s, false, c0, c1 - c0);
+      t.geom = a.geom;
+      t.n = a.n;
+      t.sc = a.sc;
+      t.ds = a.ds;
+      t.sums = w.sums + (size_t)s * steps * 2 * w.Rp;
+      t.prm = h->d_prm;
+      t.s = s;
+      t.Rp = w.Rp;
+      t.R = R;
+      t.M = 2 * steps;
+      t.n1 = steps;
+      if (C > 1) {
+        t.part = (double*)(part * sizeof(double));  // made a pointer below
+        part += (size_t)C * steps * 2 * (c1 - c0);
+      }
+      tasks.push_back(t);
+    }
+  kpm_status sa = dalloc((char**)&w.cs_tasks, tasks.size() * sizeof(ColsTask));
+  if (sa == KPM_OK) sa = dalloc(&w.cs_queue, (size_t)1);
+  if (sa == KPM_OK && part) sa = dalloc(&w.cs_part, part);
+  if (sa != KPM_OK) {
+    free_cols(w);
+    return sa;
+  }
+  for (ColsTask& t : tasks)
+    t.part = C > 1 ? (double*)((char*)w.cs_part + (size_t)t.part) : nullptr;
+  KPM_CUDA(cudaMemcpy(w.cs_tasks, tasks.data(), tasks.size() * sizeof(ColsTask),
+                      cudaMemcpyHostToDevice));
+  w.cs.C = C;
+  w.cs.ntasks = ntasks;
+  w.cs.smem = best.smem;
+  w.cs.S = S;
+  w.cs.R = R;
+  w.cs.clusters = std::min(best.clusters, ntasks);
+  return KPM_OK;
+}
+
 // Partial scratch of the column-resident form for launches of up to nprod products.
 kpm_status colres_scratch(kpm_handle_s* h, int nprod) {
   auto& w = h->work;
@@ -1083,7 +1187,8 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
   const size_t out_bytes = ((size_t)S * R * M + M) * sizeof(double);
   const bool rebuild = w.Rp != Rp || w.prec != p->precision || w.M != M ||
                        w.user_v0 != user_v0 || !w.ready || w.sums_bytes < sums_bytes ||
-                       (w.cr.C > 0 && w.cr_R != R);
+                       (w.cr.C > 0 && w.cr_R != R) ||
+                       (cols_solve_kind(h, fp32) && (w.plan_S != S || w.cr_R != R));
   // The kernel sequence of one realisation.  The first call of a shape
   // launches it directly on the caller's stream (the solve is GPU-bound, so
   // the launches hide behind it); a second call of the same shape captures it
@@ -1194,6 +1299,14 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     }
     if (dense_tc_wanted(h, fp32)) setup_dense_tc(h, Rp);
     else free_dense_tc(w);
+    w.Rp = Rp;
+    if (fp32) {
+      free_cols(w);
+    } else {
+      kpm_status sa = plan_cols_solve(h, R, S, steps);
+      if (sa != KPM_OK) return sa;
+    }
+    w.plan_S = S;
     dfree(w.ring);
     w.ring = nullptr;
     {
@@ -1291,7 +1404,14 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     }
     KPM_CUDA(launch_load_v0(fp32, h->cplx, h->n, R, Rp, src, w.v[0], st));
   }
-  if (!w.exec && w.direct_done) {
+  if (w.cs.clusters > 0) {
+    // all realisations in one launch
+    KPM_CUDA(cudaMemsetAsync(w.cs_queue, 0, sizeof(int), st));
+    KPM_CUDA(cudaEventRecord(w.ev[0], st));
+    KPM_CUDA(launch_cols(false, h->geom.dims, h->has_onsite, (const ColsTask*)w.cs_tasks,
+                         w.cs.ntasks, w.cs_queue, w.cs.clusters, w.cs.C, w.cs.smem, st));
+    KPM_CUDA(cudaEventRecord(w.ev[1], st));
+  } else if (!w.exec && w.direct_done) {
     // second call of this shape: capture the sequence once
     const uint64_t before = g_launches.load();
     KPM_CUDA(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -1309,7 +1429,7 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
       return cuda_fail(e, "capture of the moment graph");
     }
   }
-  for (int s = 0; s < S; ++s) {
+  for (int s = 0; s < S && w.cs.clusters == 0; ++s) {
     if (w.exec) {
       KPM_CUDA(cudaGraphLaunch(w.exec, st));
       g_launches.fetch_add(w.kernels_per_replay);

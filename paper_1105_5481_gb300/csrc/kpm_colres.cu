@@ -671,8 +671,13 @@ bool colres_plan(int64_t n, int dims, int ell_w, bool cplx, bool fp32, int R, Co
   }
   if (best.C == 0) return false;
   if (!forceC && best_cost >= chain_us(n, R, cplx, fp32, ell_w > 0)) return false;
+  best.us = best_cost;
   *out = best;
   return true;
+}
+
+double step_chain_us(int64_t n, int R, bool cplx, bool fp32, bool ell) {
+  return chain_us(n, R, cplx, fp32, ell);
 }
 
 size_t colres_partial_doubles(const ColresPlan& pl, int nprod) {

@@ -59,6 +59,8 @@ __host__ __device__ inline size_t colres_head_bytes(size_t vec_bytes) {
 // KPM_COLRES="0" turns the form off; KPM_COLRES="C,cpc" forces a shape (which
 // may then take several waves); KPM_COLRES_TREE set forces the shuffle tree.
 bool colres_plan(int64_t n, int dims, int ell_w, bool cplx, bool fp32, int R, ColresPlan* out);
+// Estimated microseconds per product of the chain of step launches.
+double step_chain_us(int64_t n, int R, bool cplx, bool fp32, bool ell);
 // Doubles of the partial scratch for a launch of nprod products.
 size_t colres_partial_doubles(const ColresPlan& pl, int nprod);
 // dims is that of the stencil (unused for a padded-ELL plan, pl.ell_w > 0)

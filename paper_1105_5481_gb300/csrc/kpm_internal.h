@@ -57,6 +57,7 @@ struct ColresPlan {
   int64_t P = 0;    // rows per CTA: ceil(N / C)
   size_t smem = 0;  // dynamic shared memory per CTA
   int ell_w = 0;    // 0: stencil operator; > 0: padded-ELL operator of this width
+  double us = 0.0;  // estimated microseconds per product
 };
 
 // Dense products on the bf16 tensor cores by the Ozaki splitting scheme
@@ -299,8 +300,19 @@ struct kpm_handle_s {
     // of its CTA partials
     kpm::ColresPlan cr{};
     int cr_R = 0;
+    int plan_S = 0;  // realisations the plan was made for
     double* cr_gp = nullptr;
     size_t cr_gp_doubles = 0;
+    // all S > 1 realisations as column tasks of one launch (kpm_cols.h) when
+    // cs.clusters > 0: the launch shape, the realisations, vectors and products
+    // it was made for, the tasks with their queue, and the partials' scratch
+    struct {
+      int clusters = 0, C = 0, ntasks = 0, S = 0, R = 0;
+      size_t smem = 0;
+    } cs;
+    void* cs_tasks = nullptr;
+    int* cs_queue = nullptr;
+    double* cs_part = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};  // recorded around the step chain in the graph
     bool timed = false;
   } work;

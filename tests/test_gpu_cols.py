@@ -73,3 +73,30 @@ def test_column_strips_report_divergence(K):
         with pytest.raises(K.KPMError) as e:
             K.kpm_batch_run(bt)
         assert e.value.status == K.KPM_EDIVERGE
+
+
+@pytest.mark.parametrize("L,per,onsite,R,S,M", [
+    ((10, 10, 10), (True, True, True), False, 14, 128, 32),
+    ((33, 17), (True, False), True, 3, 5, 70),
+    ((9, 8, 31), (False, True, True), True, 20, 40, 34),
+    ((3, 300), (True, True), False, 1, 700, 2),
+])
+def test_realisations_in_one_launch_match_single_solves(K, L, per, onsite, R, S, M):
+    n = int(np.prod(L))
+    on = I.onsite_disorder(8, n, 2.0) if onsite else None
+    H = O.lattice_hamiltonian(L, periodic=per, onsite=on)
+    a, b = O.rescale(*O.gershgorin(H), eps=0.01)
+    with K.kpm_create_stencil(len(L), L, periodic=per, onsite=on) as h:
+        for s0 in (0, 2):  # and twice with the same plan
+            mu, pv = K.kpm_moments(h, M, R, a, b, seed=11, S=S, s0=s0, per_vec=True)
+            assert K.kpm_testing_last_step_form(h) == "column strips"
+            np.testing.assert_allclose(mu, pv.mean(0), rtol=0, atol=1e-13)
+            for s in (0, 1, S // 2, S - 1):
+                mu_o, per_o = O.moments_doubling(H, a, b, I.rademacher_block(11, n, R, s=s0 + s), M)
+                assert np.abs(pv[s * R:(s + 1) * R] - per_o).max() <= TOL["fp64"]
+        # another S on the handle, and a single realisation that can be extended
+        mu2, pv2 = K.kpm_moments(h, M, R, a, b, seed=11, S=2, s0=2, per_vec=True)
+        assert np.abs(pv2 - pv[:2 * R]).max() <= SUMS["fp64"]
+        K.kpm_moments(h, M, R, a, b, seed=11, s0=2)
+        ext, _ = K.kpm_moments_extend(h, M + 2, R=R, per_vec=True)
+        assert np.abs(ext[:M] - pv[:R].mean(0)).max() <= 1e-12
