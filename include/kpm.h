@@ -138,8 +138,9 @@ kpm_status kpm_stencil_to_csr(const kpm_stencil_desc* desc, kpm_field field, int
 
 /* Spectral bounds (Eq. (tilde) and the text below it): the Gershgorin
  * enclosure [min_i(H_ii - sum_j|H_ij|), max_i(H_ii + sum_j|H_ij|)], tightened
- * by a lanczos_steps-step FP64 Lanczos run with full reorthogonalisation from
- * a Rademacher start vector drawn from (seed, stream 6): the extreme Ritz
+ * by a lanczos_steps-step FP64 Lanczos run with reorthogonalisation (in every
+ * step, or on large operators in the steps that need it) from a Rademacher
+ * start vector drawn from (seed, stream 6): the extreme Ritz
  * values widened by their residuals beta_k |s_k|, clamped to the Gershgorin
  * enclosure (lanczos_steps = 0 gives Gershgorin alone).  Outputs (host
  * pointers, any may be NULL): emin, emax, and the rescaling

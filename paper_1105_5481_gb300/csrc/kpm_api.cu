@@ -657,6 +657,10 @@ bool columns_in_range(const int32_t* col, int64_t nnz, int64_t n) {
 
 using namespace kpm;
 
+// Smallest dimension whose Lanczos vectors are reorthogonalised only where
+// needed.
+constexpr int64_t LANCZOS_PARTIAL_MIN_N = 1 << 16;
+
 extern "C" {
 
 const char* kpm_last_error(void) { return t_err.c_str(); }
@@ -921,11 +925,15 @@ kpm_status kpm_bounds(kpm_handle h, int lanczos_steps, double pad_eps, uint64_t 
   const int64_t len = 2 * h->n;  // flat FP64 scalars of one Lanczos vector
   double *pmin = nullptr, *pmax = nullptr, *gersh = nullptr, *out = nullptr;
   double *Q = nullptr, *y = nullptr, *part = nullptr, *part_loc = nullptr, *coef = nullptr,
-         *alpha = nullptr, *beta = nullptr;
+         *alpha = nullptr, *beta = nullptr, *omega = nullptr;
+  int* flag = nullptr;
+  // partial reorthogonalisation where the Gram-Schmidt passes outweigh the
+  // launches that decide on them (kpm_aux.cu)
+  const bool partial = h->n >= LANCZOS_PARTIAL_MIN_N;
   kpm_status st_ = KPM_OK;
   auto cleanup = [&]() {
     dfree(pmin); dfree(pmax); dfree(gersh); dfree(out); dfree(Q); dfree(y); dfree(part);
-    dfree(part_loc); dfree(coef); dfree(alpha); dfree(beta);
+    dfree(part_loc); dfree(coef); dfree(alpha); dfree(beta); dfree(omega); dfree(flag);
   };
 #define KPM_TRY(call)                                \
   do {                                               \
@@ -954,7 +962,8 @@ kpm_status kpm_bounds(kpm_handle h, int lanczos_steps, double pad_eps, uint64_t 
   if (k > 0) {
     if ((st_ = dalloc(&Q, (size_t)(k + 1) * len)) || (st_ = dalloc(&y, len)) ||
         (st_ = dalloc(&part, (size_t)nblk * 2 * (k + 1))) || (st_ = dalloc(&part_loc, (size_t)nblk * 4)) ||
-        (st_ = dalloc(&coef, 2 * (k + 1)))) {
+        (st_ = dalloc(&coef, 2 * (k + 1))) ||
+        (partial && ((st_ = dalloc(&omega, 3 * (size_t)(k + 1))) || (st_ = dalloc(&flag, (size_t)k))))) {
       cudaStreamSynchronize(st);
       cleanup();
       return st_;
@@ -978,10 +987,15 @@ kpm_status kpm_bounds(kpm_handle h, int lanczos_steps, double pad_eps, uint64_t 
       sa.partial = nullptr;
       KPM_TRY(launch_op(h, false, MODE_SPMV, sa, LaunchCfg{block, grid}, st));
       // three-term step against q_j, q_{j-1}, then one full Gram-Schmidt pass
+      // (partial: where the step is flagged)
       KPM_TRY(launch_lz_local_dots(h->cplx, h->n, Q, len, j, y, part_loc, nblk, st));
-      KPM_TRY(launch_lz_reorth_dots(h->cplx, h->n, Q, len, j, part_loc, y, part, alpha, nblk, st));
-      KPM_TRY(launch_dots_final(part, nblk, j, coef, st));
-      KPM_TRY(launch_lz_update_norm(h->cplx, h->n, Q, len, j, coef, y, part, nblk, st));
+      if (partial) {
+        KPM_TRY(launch_lz_three_term(h->cplx, h->n, Q, len, j, part_loc, y, part, alpha, nblk, st));
+        KPM_TRY(launch_lz_omega(j, k, nblk, part, alpha, beta, omega, flag, st));
+      }
+      KPM_TRY(launch_lz_reorth_dots(h->cplx, h->n, Q, len, j, part_loc, y, part, alpha, nblk, flag, st));
+      KPM_TRY(launch_dots_final(part, nblk, j, coef, flag, st));
+      KPM_TRY(launch_lz_update_norm(h->cplx, h->n, Q, len, j, coef, y, part, nblk, flag, st));
       KPM_TRY(launch_lanczos_next(h->n, y, part, nblk, beta, j, Q + (size_t)(j + 1) * len, st));
     }
   }

@@ -148,11 +148,17 @@ cudaError_t launch_lz_local_dots(bool cplx, int64_t n, const double* Q, int64_t 
                                 const double* y, double* part_loc, int nblk, cudaStream_t st);
 cudaError_t launch_lz_reorth_dots(bool cplx, int64_t n, const double* Q, int64_t ldq, int j,
                                   const double* part_loc, double* y, double* part, double* alpha,
-                                  int nblk, cudaStream_t st);
-cudaError_t launch_dots_final(const double* part, int nblk, int j, double* out, cudaStream_t st);
+                                  int nblk, const int* flag, cudaStream_t st);
+cudaError_t launch_lz_three_term(bool cplx, int64_t n, const double* Q, int64_t ldq, int j,
+                                 const double* part_loc, double* y, double* part, double* alpha,
+                                 int nblk, cudaStream_t st);
+cudaError_t launch_lz_omega(int j, int k, int nblk, const double* part, const double* alpha,
+                            const double* beta, double* w, int* flag, cudaStream_t st);
+cudaError_t launch_dots_final(const double* part, int nblk, int j, double* out, const int* flag,
+                              cudaStream_t st);
 cudaError_t launch_lz_update_norm(bool cplx, int64_t n, const double* Q, int64_t ldq, int j,
                                   const double* coef, double* y, double* part, int nblk,
-                                  cudaStream_t st);
+                                  const int* flag, cudaStream_t st);
 cudaError_t launch_lanczos_next(int64_t n, const double* y, const double* part, int nblk,
                                 double* beta, int j, double* qnext, cudaStream_t st);
 cudaError_t launch_tridiag_bounds(const double* alpha, const double* beta, int m,
