@@ -198,40 +198,55 @@ __global__ void reduce_ring_kernel(const double* __restrict__ ring, int ring_slo
 
 __global__ void advance_realisation_kernel(RunParams* prm) { prm->s += 1; }
 
-// Doubling identities per vector, then the average over all S*R vectors.
-__global__ void finalize_pervec_kernel(const double* __restrict__ sums, int S, int steps, int R,
-                                       int Rp, int64_t n, int M, double* per_vec, RunParams* prm) {
-  const int64_t total = (int64_t)S * R * steps;
-  const int w = 2 * Rp;
-  const double inv_n = 1.0 / (double)n;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int step = (int)(e % steps);
-    const int64_t sr = e / steps;
-    const int r = (int)(sr % R), s = (int)(sr / R);
-    const double* base = sums + (size_t)s * steps * w;
-    const double mu0 = base[r] * inv_n, mu1 = base[Rp + r] * inv_n;
-    double me, mo;
-    if (step == 0) {
-      me = mu0;
-      mo = mu1;
-    } else {
-      me = 2.0 * base[(size_t)step * w + r] * inv_n - mu0;
-      mo = 2.0 * base[(size_t)step * w + Rp + r] * inv_n - mu1;
+// Per-vector moments from the per-step sums and their mean over all S R
+// vectors: mu_{2n} = 2 A_n / N - mu_0, mu_{2n+1} = 2 B_n / N - mu_1.  A CTA
+// takes 8 products; warp q its product q, lane l the vectors l, l + 32, ...
+// (the sums of a product lie along the vectors), and two threads per product
+// add the lanes' subtotals in lane order.  One launch, where the mean used to
+// be a second one behind the per-vector values (2.5 us of a small solve) that
+// walked all S R vectors in one thread per moment.
+constexpr int FIN_STEPS = 8;
+__global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* __restrict__ sums, int S,
+                                                                  int steps, int R, int Rp, int64_t n,
+                                                                  int M, double* per_vec, double* mu,
+                                                                  RunParams* prm) {
+  __shared__ double sub[FIN_STEPS][2][33];
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  const int step = blockIdx.x * FIN_STEPS + q;
+  const int w = 2 * Rp, cols = S * R;
+  const double inv_n = 1.0 / (double)n, lim = 1.0 + 1e-6;
+  double se = 0.0, so = 0.0;
+  bool bad = false;
+  if (step < steps) {
+    for (int sr = lane; sr < cols; sr += 32) {
+      const int s = sr / R, r = sr - s * R;
+      const double* base = sums + (size_t)s * steps * w;
+      const double mu0 = base[r] * inv_n, mu1 = base[Rp + r] * inv_n;
+      double me = mu0, mo = mu1;
+      if (step > 0) {
+        me = 2.0 * base[(size_t)step * w + r] * inv_n - mu0;
+        mo = 2.0 * base[(size_t)step * w + Rp + r] * inv_n - mu1;
+      }
+      double* pv = per_vec + (size_t)sr * M + 2 * step;
+      pv[0] = me;
+      pv[1] = mo;
+      bad |= !(fabs(me) <= lim) || !(fabs(mo) <= lim);
+      se += me;
+      so += mo;
     }
-    per_vec[(size_t)sr * M + 2 * step] = me;
-    per_vec[(size_t)sr * M + 2 * step + 1] = mo;
-    const double lim = 1.0 + 1e-6;
-    if (!(fabs(me) <= lim) || !(fabs(mo) <= lim)) atomicOr(&prm->flags, 1);
   }
-}
-
-__global__ void finalize_mean_kernel(const double* __restrict__ per_vec, int cols, int M,
-                                     double* mu) {
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int c = 0; c < cols; ++c) acc += per_vec[(size_t)c * M + m];
-    mu[m] = acc / (double)cols;
+  if (bad) atomicOr(&prm->flags, 1);
+  sub[q][0][lane] = se;
+  sub[q][1][lane] = so;
+  __syncthreads();
+  if (threadIdx.x < 2 * FIN_STEPS) {
+    const int qq = threadIdx.x >> 1, c = threadIdx.x & 1, st = blockIdx.x * FIN_STEPS + qq;
+    if (st < steps) {
+      double acc = 0.0;
+      const int nl = min(32, cols);
+      for (int l = 0; l < nl; ++l) acc += sub[qq][c][l];
+      mu[2 * st + c] = acc / (double)cols;
+    }
   }
 }
 
@@ -876,20 +891,23 @@ __device__ __forceinline__ double damping(int n, int M, int kernel, double lambd
 // clock; a 256-thread block of cos/sin on one SM took about 12 us for M = 256).
 constexpr int FP64_SPREAD = 32;
 
-__global__ void dos_coef_kernel(const double* __restrict__ mu, int M, int kernel, double lambda,
-                                double* coef) {
-  const double q = M_PI / (double)(M + 1);
-  const double cotq = cos(q) / sin(q);
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < M; n += gridDim.x * blockDim.x)
-    coef[n] = (n == 0 ? 1.0 : 2.0) * damping(n, M, kernel, lambda, cotq) * (mu ? mu[n] : 1.0);
-}
-
-// table[j] = cos(pi j / (2K)), j = 0 .. 4K-1 (exact argument reduction for the DCT)
-__global__ void cos_table_kernel(int K, double* table) {
-  const int64_t n4 = 4LL * K;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n4;
-       j += (int64_t)gridDim.x * blockDim.x)
-    table[j] = cospi((double)j / (2.0 * (double)K));
+// The damped coefficients coef[n] = c_n g_n mu_n (mu NULL: 1) and the cosine
+// table[j] = cos(pi j / (2K)), j = 0 .. 4K-1 (exact argument reduction for the
+// sums): independent of each other, one launch.
+__global__ void dos_prep_kernel(const double* __restrict__ mu, int M, int kernel, double lambda,
+                                double* coef, int K, double* table) {
+  const int64_t total = M + 4LL * K;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    if (e < M) {
+      const int n = (int)e;
+      const double q = M_PI / (double)(M + 1);
+      const double cotq = cos(q) / sin(q);
+      coef[n] = (n == 0 ? 1.0 : 2.0) * damping(n, M, kernel, lambda, cotq) * (mu ? mu[n] : 1.0);
+    } else {
+      table[e - M] = cospi((double)(e - M) / (2.0 * (double)K));
+    }
+  }
 }
 
 // T lanes per node k (T a power of two <= 32): lane `sub` adds the terms
@@ -1301,12 +1319,8 @@ cudaError_t launch_advance_realisation(RunParams* prm, cudaStream_t st) {
 
 cudaError_t launch_finalize(const double* sums, int S, int steps, int R, int Rp, int64_t n, int M,
                             double* per_vec, double* mu, RunParams* prm, cudaStream_t st) {
-  const unsigned g = blocks_for((int64_t)S * R * steps, 256);
-  finalize_pervec_kernel<<<g, 256, 0, st>>>(sums, S, steps, R, Rp, n, M, per_vec, prm);
-  counted(cudaSuccess);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  finalize_mean_kernel<<<blocks_for(M, 128), 128, 0, st>>>(per_vec, S * R, M, mu);
+  finalize_kernel<<<(unsigned)((steps + FIN_STEPS - 1) / FIN_STEPS), FIN_STEPS * 32, 0, st>>>(
+      sums, S, steps, R, Rp, n, M, per_vec, mu, prm);
   return counted(cudaGetLastError());
 }
 
@@ -1428,13 +1442,10 @@ cudaError_t launch_stats(const double* pv, int nvec, int M, double a, double b, 
     if (e != cudaSuccess) return e;
   }
   if (!E && !rmean && !rerr) return cudaSuccess;
-  dos_coef_kernel<<<blocks_for(M, FP64_SPREAD), FP64_SPREAD, 0, st>>>(nullptr, M, kernel, lambda, g);
+  dos_prep_kernel<<<blocks_for(M + 4LL * K, FP64_SPREAD), FP64_SPREAD, 0, st>>>(nullptr, M, kernel, lambda, g, K,
+                                                                             table);
   counted(cudaSuccess);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  cos_table_kernel<<<blocks_for(4LL * K, FP64_SPREAD), FP64_SPREAD, 0, st>>>(K, table);
-  counted(cudaSuccess);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (rmean || rerr) {
     if (const int N1 = dos_split(K, M)) {
@@ -1471,13 +1482,10 @@ cudaError_t launch_green(const double* mu, int M, double a, double b, int K, int
                          cudaStream_t st) {
   double* coef = work;
   double* table = work + M;
-  dos_coef_kernel<<<blocks_for(M, FP64_SPREAD), FP64_SPREAD, 0, st>>>(mu, M, kernel, lambda, coef);
+  dos_prep_kernel<<<blocks_for(M + 4LL * K, FP64_SPREAD), FP64_SPREAD, 0, st>>>(mu, M, kernel, lambda, coef, K,
+                                                                             table);
   counted(cudaSuccess);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  cos_table_kernel<<<blocks_for(4LL * K, FP64_SPREAD), FP64_SPREAD, 0, st>>>(K, table);
-  counted(cudaSuccess);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   green_kernel<<<blocks_for(32LL * K, 256), 256, 0, st>>>(coef, M, a, b, K, table, E, g_re, g_im);
   return counted(cudaGetLastError());
@@ -1504,13 +1512,10 @@ cudaError_t launch_dos(const double* mu, int M, double a, double b, int K, int k
                        double lambda, double* E, double* rho, double* work, cudaStream_t st) {
   double* coef = work;
   double* table = work + M;
-  dos_coef_kernel<<<blocks_for(M, FP64_SPREAD), FP64_SPREAD, 0, st>>>(mu, M, kernel, lambda, coef);
+  dos_prep_kernel<<<blocks_for(M + 4LL * K, FP64_SPREAD), FP64_SPREAD, 0, st>>>(mu, M, kernel, lambda, coef, K,
+                                                                             table);
   counted(cudaSuccess);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  cos_table_kernel<<<blocks_for(4LL * K, FP64_SPREAD), FP64_SPREAD, 0, st>>>(K, table);
-  counted(cudaSuccess);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // lanes per node: enough threads for about 4 warps per SM, at most a warp
   int T = 1;
