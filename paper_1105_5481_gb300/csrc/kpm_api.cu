@@ -5,6 +5,7 @@
 // of kpm_step_*.cu and kpm_aux.cu.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -21,6 +22,11 @@
 #include "kpm_internal.h"
 
 namespace kpm {
+
+// Largest operators whose FP64 vectors go into 64-bit fixed point: the unit is
+// 2^-52 or finer for real fields, 2^-51 for complex ones (whose rows have four
+// times the terms, each with its rounding, on the FP64 pipe).
+constexpr int64_t FIXED_MAX_N_REAL = 1 << 18, FIXED_MAX_N_CPLX = 1 << 20;
 
 // vector columns per chunk (FP32: 32-byte chunks; FP64: 16-byte chunks)
 int vec_per_chunk(bool fp32, bool cplx) { return fp32 ? (cplx ? 4 : 8) : (cplx ? 1 : 2); }
@@ -274,6 +280,7 @@ cudaError_t launch_op(const kpm_handle_s* h, bool fp32, StepMode mode, const Ste
     if (h->work.dtc && mode != MODE_SPMV) return launch_dense_tc_step(*h->work.dtc, mode, a, cfg, st);
     return launch_dense_step(h->cplx, mode, a, cfg, st);
   }
+  if (a.fixq > 0) return launch_step_i64(h->stencil, h->cplx, mode, a, cfg, st);
   return launch_step(h->stencil, fp32, h->cplx, mode, a, cfg, st);
 }
 
@@ -336,7 +343,8 @@ void plan_grid(const kpm_handle_s* h, bool fp32, StepArgs& a, int* block, int* g
   while (blk / 2 >= std::max(32, G) && (h->n * G + blk - 1) / blk < h->num_sms) blk /= 2;
   const int spi = blk / G;
   int occ = fp32 ? occ_step_f32(h->stencil, h->cplx, a, blk)
-                 : occ_step_f64(h->stencil, h->cplx, a, blk);
+          : a.fixq > 0 ? occ_step_i64(h->stencil, h->cplx, a, blk)
+                       : occ_step_f64(h->stencil, h->cplx, a, blk);
   occ = std::max(1, std::min(occ, 8));
   a.line_len = 0;
   a.lines = 0;
@@ -487,6 +495,8 @@ void destroy_handle(kpm_handle_s* h) {
   cudaSetDevice(h->device);
   cudaDeviceSynchronize();
   free_work(h);
+  dfree(h->d_hs_fix);
+  dfree(h->d_ds_fix);
   dfree(h->d_onsite);
   dfree(h->d_hop);
   dfree(h->d_rowptr);
@@ -1047,12 +1057,87 @@ ColresArgs colres_args(const kpm_handle_s* h, int R, int n0, int n1, int steps, 
   return c;
 }
 
+// Calls whose step chain may run in 64-bit fixed point (kpm_fixed.cuh): FP64
+// vectors on a stencil or CSR operator of up to FIXED_MAX_N_* rows, with a start
+// block made by the library (its norm is sqrt(N)).  Faster from the smallest
+// chains on (measured at M = 256, 1 to 64 columns: 1.0 to 1.3 times at 1,500
+// rows, 1.1 to 2.4 at 8,000 to 300,000).  KPM_FIXED=0 keeps the FP64 pipe.
+bool fixed_kind(const kpm_handle_s* h, bool fp32, const kpm_params* p) {
+  if (fp32 || h->dense || h->n > (h->cplx ? FIXED_MAX_N_CPLX : FIXED_MAX_N_REAL) || p->user_v0) return false;
+  const char* env = getenv("KPM_FIXED");
+  return !(env && env[0] == '0');
+}
+
+// The range of the handle's coefficients, for fixed_unit (once per handle;
+// synchronises).
+kpm_status ensure_range(kpm_handle_s* h) {
+  if (h->ranged) return KPM_OK;
+  const int nblk = (int)std::min<int64_t>((h->n + 255) / 256, 2 * (int64_t)h->num_sms);
+  double* w = nullptr;
+  kpm_status st = dalloc(&w, 3 * (size_t)nblk + 4);
+  if (st != KPM_OK) return st;
+  double out[4], *o = w + 3 * (size_t)nblk;
+  cudaError_t e = launch_coef_range(h->cplx, h->n, h->stencil ? &h->geom : nullptr, h->d_onsite,
+                                    h->d_hop, h->t_re, h->t_im, h->d_rowptr, h->d_val, w, nblk, 0);
+  if (e == cudaSuccess) e = launch_minmax_final(w, w + nblk, nblk, o, 0);
+  if (e == cudaSuccess) e = launch_minmax_final(w + 2 * nblk, w + 2 * nblk, nblk, o + 2, 0);
+  if (e == cudaSuccess) e = cudaMemcpy(out, o, sizeof(out), cudaMemcpyDeviceToHost);
+  dfree(w);
+  if (e != cudaSuccess) return cuda_fail(e, "range of the coefficients");
+  h->range[0] = out[0];
+  h->range[1] = out[1];
+  h->range[2] = out[3];
+  h->ranged = true;
+  return KPM_OK;
+}
+
+// The unit 2^-q of a call of that kind with rescaling (a, b), or 0 where its
+// coefficients leave the format's range: a scaled hopping or diagonal of 7, or
+// a row of 15 in sum of components.  (a, b) that enclose the spectrum give
+// about 2 to 6.
+int fixed_unit(const kpm_handle_s* h, double a, double b) {
+  const double s = 2.0 / a, t = h->range[2];
+  const double d = std::max(fabs(h->range[1] - b), fabs(h->range[0] - b));
+  if (!(s * t <= 7.0) || !(s * d <= 7.0) || !(s * (t + d) <= 15.0)) return 0;
+  int lg = 0;
+  while (((int64_t)1 << lg) < h->n) ++lg;
+  return 61 - (lg + 1) / 2;
+}
+
+// The unit of the column tasks (kpm_cols.cuh): one bit less, because they sum the
+// neighbours before they multiply; 0 where that would be coarser than 2^-52.
+int cols_unit(int q) { return q >= 53 ? q - 1 : 0; }
+
+// Scalars of the hoppings (stencil) or entries (padded ELL, CSR) of slot 0.
+int64_t fixed_entries(const kpm_handle_s* h) {
+  const int c = h->cplx ? 2 : 1;
+  if (h->stencil) return h->has_hop ? h->n * h->geom.dims * c : 0;
+  return (h->ell_w > 0 ? h->n * h->ell_w : h->nnz) * c;
+}
+
+// Buffers of the operator's fixed-point copies.
+kpm_status ensure_fixed(kpm_handle_s* h) {
+  char *ph = nullptr, *pd = nullptr;
+  kpm_status st = KPM_OK;
+  if (fixed_entries(h) > 0 && !h->d_hs_fix) {
+    if ((st = dalloc(&ph, (size_t)fixed_entries(h) * 8)) != KPM_OK) return st;
+    h->d_hs_fix = ph;
+  }
+  if (h->has_onsite && !h->d_ds_fix) {
+    if ((st = dalloc(&pd, (size_t)h->n * 8)) != KPM_OK) return st;
+    h->d_ds_fix = pd;
+  }
+  h->fix_ok = false;
+  return KPM_OK;
+}
+
 // Several realisations of a 2D or 3D stencil of uniform real hopping with FP64
 // vectors: their S R columns are independent recursions, so all of them go as
 // column tasks into one persistent launch (kpm_cols.h) when that is estimated
 // faster than S solves one after the other.  A single small realisation leaves
 // most of the FP64 pipes idle (10^3 cube, 14 vectors, 128 realisations, M =
-// 256: 17.7 ms one after the other, 4.9 ms in one launch, 4.2 of it FP64 work).  FP32 vectors keep the
+// 256: 17.7 ms one after the other, 4.9 ms in one launch on the FP64 pipe, 2.0
+// in fixed point).  FP32 vectors keep the
 // solves in turn: their compensated dots depend on the form's sum order.
 bool cols_solve_kind(const kpm_handle_s* h, bool fp32) {
   return !fp32 && h->stencil && !h->cplx && !h->has_hop && (h->geom.dims == 2 || h->geom.dims == 3);
@@ -1060,7 +1145,7 @@ bool cols_solve_kind(const kpm_handle_s* h, bool fp32) {
 
 // Plans the launch for the current buffers; leaves w.cs.clusters 0 where the
 // form does not apply.
-kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps) {
+kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps, int fixq) {
   auto& w = h->work;
   free_cols(w);
   if (S < 2 || !cols_solve_kind(h, false) || getenv("KPM_COLRES")) return KPM_OK;
@@ -1087,7 +1172,9 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps) {
     }
     if (t.clusters < 1) continue;
     const int64_t tasks = (int64_t)S * ((R + t.width - 1) / t.width);
-    t.us = (double)((tasks + t.clusters - 1) / t.clusters) * (t.s.us_fixed + t.width * t.s.us_col);
+    // fixed point: about 90 issue slots per site against 64 per FP64 instruction
+    t.us = (double)((tasks + t.clusters - 1) / t.clusters) *
+           (t.s.us_fixed + t.width * t.s.us_col * (fixq > 0 ? 0.25 : 1.0));
     if (t.us < best.us) best = t;
   }
   if (best.s.C == 0) return KPM_OK;
@@ -1104,7 +1191,8 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps) {
       t.geom = a.geom;
       t.n = a.n;
       t.sc = a.sc;
-      t.ds = a.ds;
+      t.ds = fixq > 0 && h->has_onsite ? h->d_ds_fix : a.ds;
+      t.fixq = fixq;
       t.sums = w.sums + (size_t)s * steps * 2 * w.Rp;
       t.prm = h->d_prm;
       t.s = s;
@@ -1123,6 +1211,7 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps) {
   if (sa == KPM_OK && part) sa = dalloc(&w.cs_part, part);
   if (sa != KPM_OK) {
     free_cols(w);
+    if (sa == KPM_ENOMEM) return KPM_OK;  // the solves in turn need none of it
     return sa;
   }
   for (ColsTask& t : tasks)
@@ -1130,6 +1219,7 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps) {
   KPM_CUDA(cudaMemcpy(w.cs_tasks, tasks.data(), tasks.size() * sizeof(ColsTask),
                       cudaMemcpyHostToDevice));
   w.cs.C = C;
+  w.cs.fixq = fixq;
   w.cs.ntasks = ntasks;
   w.cs.smem = best.smem;
   w.cs.S = S;
@@ -1197,12 +1287,19 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
   kpm_status s_ = ensure_scaled(h, slot, fp32);
   if (s_ != KPM_OK) return s_;
 
+  // the step chain in fixed point, decided when it is planned and again when
+  // a call's kind or (a, b) would decide otherwise
+  const bool fix_kind = fixed_kind(h, fp32, p);
+  const int unit_now = fix_kind && h->ranged ? fixed_unit(h, p->a, p->b) : 0;
   const size_t sums_bytes = (size_t)S * steps * 2 * Rp * sizeof(double);
   const size_t out_bytes = ((size_t)S * R * M + M) * sizeof(double);
   const bool rebuild = w.Rp != Rp || w.prec != p->precision || w.M != M ||
                        w.user_v0 != user_v0 || !w.ready || w.sums_bytes < sums_bytes ||
                        (w.cr.C > 0 && w.cr_R != R) ||
-                       (cols_solve_kind(h, fp32) && (w.plan_S != S || w.cr_R != R));
+                       (cols_solve_kind(h, fp32) && (w.plan_S != S || w.cr_R != R)) ||
+                       (!h->dense && w.cr.C == 0 && w.cs.clusters == 0 &&
+                        (w.proto.fixq > 0) != (h->ranged ? unit_now > 0 && !w.fix_off : fix_kind && w.proto.fixq > 0)) ||
+                       (w.cs.clusters > 0 && w.cs.fixq != (w.fix_off ? 0 : cols_unit(unit_now)));
   // The kernel sequence of one realisation.  The first call of a shape
   // launches it directly on the caller's stream (the solve is GPU-bound, so
   // the launches hide behind it); a second call of the same shape captures it
@@ -1228,6 +1325,8 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
       return e;
     }
     if (!user_v0) e = launch_rng_init(fp32, h->cplx, h->n, Rp, h->d_prm, w.v[0], cs);
+    if (e == cudaSuccess && !user_v0 && w.proto.fixq > 0)
+      e = launch_to_fixed(h->n * Rp * (h->cplx ? 2 : 1), w.proto.fixq, w.v[0], cs);
     StepArgs a = w.proto;
     if (e == cudaSuccess) e = rec(w.ev[0]);
     if (e == cudaSuccess) {
@@ -1269,6 +1368,7 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     // later call may take the old one (an allocation failing half way leaves
     // the handle to rebuild on its next call)
     w.ready = false;
+    w.fix_off = false;
     const size_t vbytes = (size_t)h->n * Rp * elem_bytes(fp32, h->cplx);
     if (w.vbytes < vbytes) {
       dfree(w.v[0]);
@@ -1317,10 +1417,36 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     if (fp32) {
       free_cols(w);
     } else {
-      kpm_status sa = plan_cols_solve(h, R, S, steps);
+      int q = 0;
+      kpm_status sa = KPM_OK;
+      if (S > 1 && fix_kind && cols_solve_kind(h, fp32)) {
+        sa = ensure_range(h);
+        if (sa == KPM_OK && (q = cols_unit(fixed_unit(h, p->a, p->b))) > 0) sa = ensure_fixed(h);
+        if (sa == KPM_ENOMEM) {
+          w.fix_off = true;
+          q = 0;
+          sa = KPM_OK;
+        }
+      }
+      if (sa == KPM_OK) sa = plan_cols_solve(h, R, S, steps, q);
       if (sa != KPM_OK) return sa;
     }
     w.plan_S = S;
+    if (fix_kind && !w.fix_off && w.cr.C == 0 && w.cs.clusters == 0) {
+      // (without memory for the operator's second copy: the FP64 pipe)
+      kpm_status sa = ensure_range(h);
+      const int q = sa == KPM_OK ? fixed_unit(h, p->a, p->b) : 0;
+      if (q > 0) sa = ensure_fixed(h);
+      if (sa == KPM_ENOMEM) w.fix_off = true;
+      else if (sa != KPM_OK) return sa;
+      else if (q > 0) {
+        w.proto.fixq = q;
+        if (!h->stencil) w.proto.vals = h->d_hs_fix;
+        else if (h->has_hop) w.proto.hs = h->d_hs_fix;
+        if (h->has_onsite) w.proto.ds = h->d_ds_fix;
+        plan_grid(h, fp32, w.proto, &block, &grid);
+      }
+    }
     dfree(w.ring);
     w.ring = nullptr;
     {
@@ -1371,11 +1497,18 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
   if (!(h->scaled_ok[slot] && h->scaled_a[slot] == p->a && h->scaled_b[slot] == p->b &&
         h->scaled_st[slot] == stream)) {
     h->scaled_ok[slot] = false;
+    if (slot == 0) h->fix_ok = false;
     KPM_CUDA(prescale(h, slot, fp32, false, st));
     h->scaled_ok[slot] = true;
     h->scaled_a[slot] = p->a;
     h->scaled_b[slot] = p->b;
     h->scaled_st[slot] = stream;
+  }
+  if ((w.proto.fixq > 0 || (w.cs.clusters > 0 && w.cs.fixq > 0)) && !h->fix_ok) {
+    if (const int64_t m = fixed_entries(h))
+      KPM_CUDA(launch_to_fix_coef(m, h->stencil ? h->d_hs[0] : h->d_vals[0], h->d_hs_fix, st));
+    if (h->has_onsite) KPM_CUDA(launch_to_fix_coef(h->n, h->d_ds[0], h->d_ds_fix, st));
+    h->fix_ok = true;
   }
   if (w.dtc) KPM_CUDA(launch_dense_tc_slice_rows(*w.dtc, (const double*)h->d_vals[slot], st));
   if (sb.kind != START_RANDOM) {
@@ -1398,6 +1531,8 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
                              pb, cudaMemcpyHostToDevice, st));
     KPM_CUDA(launch_start_block(fp32, h->cplx, sb.kind, h->n, R, Rp, w.sb_dev, h->geom,
                                 w.v[0], st));
+    if (w.proto.fixq > 0)
+      KPM_CUDA(launch_to_fixed(h->n * Rp * (h->cplx ? 2 : 1), w.proto.fixq, w.v[0], st));
   } else if (user_v0) {
     const size_t vb = (size_t)h->n * R * (h->cplx ? 2 : 1) * sizeof(double);
     const double* src = (const double*)p->user_v0;
@@ -1639,7 +1774,9 @@ kpm_status kpm_moments_extend(kpm_handle h, int M, double* mu, double* mu_per_ve
   prm.S = 1;
   prm.M = M;
   prm.flags = 0;
-  KPM_CUDA(cudaMemcpyAsync(h->d_prm, &prm, sizeof(prm), cudaMemcpyHostToDevice, st));
+  // (a fixed-point value out of range in an earlier call stays flagged)
+  KPM_CUDA(cudaMemcpyAsync(h->d_prm, &prm, w.proto.fixq > 0 ? offsetof(RunParams, flags) : sizeof(prm),
+                           cudaMemcpyHostToDevice, st));
   // the same step launches as the uninterrupted chain: product n reads v_n
   // from v[n & 1] and writes v_{n+1} over v_{n-1}; the ring is reduced at the
   // same step boundaries, so the sums equal those of a single call with this M

@@ -90,7 +90,10 @@ struct StepArgs {
   int tma_prefetch;       // >= 0: L2 prefetch of the off-tile neighbour rows of the tile
                           // that many tiles ahead; < 0: none
   int tma_stall;          // testing aid: the producer issues no copy (the waits run out)
-  int* err;               // bit 2 set by a bounded wait that ran out (may be NULL)
+  int* err;               // bit 2 set by a bounded wait that ran out (may be NULL); bit 3 by a
+                          // fixed-point value out of range
+  int fixq;               // > 0: FP64 vectors held as 64-bit fixed point, 2^-fixq the unit
+                          // (kpm_fixed.cuh)
 };
 
 struct LaunchCfg {

@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* 
   const int step = blockIdx.x * FIN_STEPS + q;
   const int w = 2 * Rp, cols = S * R;
   const double inv_n = 1.0 / (double)n, lim = 1.0 + 1e-6;
+  const bool out_of_range = (prm->flags & 8) != 0;  // a fixed-point value left its range
   double se = 0.0, so = 0.0;
   bool bad = false;
   if (step < steps) {
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* 
         me = 2.0 * base[(size_t)step * w + r] * inv_n - mu0;
         mo = 2.0 * base[(size_t)step * w + Rp + r] * inv_n - mu1;
       }
+      if (out_of_range) me = mo = NAN;
       double* pv = per_vec + (size_t)sr * M + 2 * step;
       pv[0] = me;
       pv[1] = mo;
@@ -349,6 +351,71 @@ __global__ void gershgorin_csr_kernel(bool cplx, int64_t n, const int64_t* __res
     pmin[blockIdx.x] = smin[0];
     pmax[blockIdx.x] = smax[0];
   }
+}
+
+// Range of the coefficients a row's product uses, for the fixed-point step: the
+// least and greatest on-site energy (0 without), and the greatest sum of the
+// components' magnitudes over a row's bonds (CSR: over its entries), as the
+// step applies them: a periodic side of length 1 or 2 has both its bonds.
+__device__ __forceinline__ void coef_range_out(double lo, double hi, double t, double* part, int nblk) {
+  __shared__ double s[3][256];
+  const int x = threadIdx.x;
+  s[0][x] = lo;
+  s[1][x] = hi;
+  s[2][x] = t;
+  __syncthreads();
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    if (x < o) {
+      s[0][x] = fmin(s[0][x], s[0][x + o]);
+      s[1][x] = fmax(s[1][x], s[1][x + o]);
+      s[2][x] = fmax(s[2][x], s[2][x + o]);
+    }
+    __syncthreads();
+  }
+  if (x < 3) part[(size_t)x * nblk + blockIdx.x] = s[x][0];
+}
+
+__global__ void coef_range_stencil_kernel(bool cplx, int64_t n, StencilGeom g,
+                                          const double* __restrict__ onsite,
+                                          const double* __restrict__ hop, double t_re, double t_im,
+                                          double* part) {
+  double lo = INFINITY, hi = -INFINITY, t = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const double on = onsite ? onsite[i] : 0.0;
+    lo = fmin(lo, on);
+    hi = fmax(hi, on);
+    auto mag = [&](int64_t site, int d) {
+      const size_t e = (size_t)site * g.dims + d;
+      if (!hop) return fabs(t_re) + fabs(t_im);
+      return cplx ? fabs(hop[2 * e]) + fabs(hop[2 * e + 1]) : fabs(hop[e]);
+    };
+    double sum = 0.0;
+    unsigned rem = (unsigned)i;
+    for (int d = 0; d < g.dims; ++d) {
+      const int L = g.L[d], st = g.stride[d];
+      const int x = (int)(rem % (unsigned)L);
+      rem /= (unsigned)L;
+      const bool per = g.periodic[d] != 0;
+      if (x + 1 < L || per) sum += mag(i, d);
+      if (x > 0 || per) sum += mag(x > 0 ? i - st : i + (int64_t)(L - 1) * st, d);
+    }
+    t = fmax(t, sum);
+  }
+  coef_range_out(lo, hi, t, part, gridDim.x);
+}
+
+__global__ void coef_range_csr_kernel(bool cplx, int64_t n, const int64_t* __restrict__ rowptr,
+                                      const double* __restrict__ val, double* part) {
+  double t = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    double sum = 0.0;
+    for (int64_t k = rowptr[i]; k < rowptr[i + 1]; ++k)
+      sum += cplx ? fabs(val[2 * k]) + fabs(val[2 * k + 1]) : fabs(val[k]);
+    t = fmax(t, sum);
+  }
+  coef_range_out(0.0, 0.0, t, part, gridDim.x);
 }
 
 __global__ void minmax_final_kernel(const double* pmin, const double* pmax, int nblk, double* out) {
@@ -1337,6 +1404,14 @@ cudaError_t launch_gershgorin_csr(bool cplx, int64_t n, const int64_t* rowptr, c
                                   const double* val, double* part_min, double* part_max, int nblk,
                                   cudaStream_t st) {
   gershgorin_csr_kernel<<<nblk, 256, 0, st>>>(cplx, n, rowptr, col, val, part_min, part_max);
+  return counted(cudaGetLastError());
+}
+
+cudaError_t launch_coef_range(bool cplx, int64_t n, const StencilGeom* g, const double* onsite,
+                              const double* hop, double t_re, double t_im, const int64_t* rowptr,
+                              const double* val, double* part, int nblk, cudaStream_t st) {
+  if (g) coef_range_stencil_kernel<<<nblk, 256, 0, st>>>(cplx, n, *g, onsite, hop, t_re, t_im, part);
+  else coef_range_csr_kernel<<<nblk, 256, 0, st>>>(cplx, n, rowptr, val, part);
   return counted(cudaGetLastError());
 }
 

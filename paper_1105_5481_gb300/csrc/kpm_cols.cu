@@ -23,13 +23,13 @@ static size_t cols_bytes(const ColsShape& s, bool fp32, int ncol, int kb) {
     return (size_t)3 * ((s.height * (COLS_THREADS + 1) + 3) / 4 * 4) * 4 +
            (size_t)2 * kb * ncol * s.ranks * 16 * 8 + s.table;
   return ((2 * (size_t)ncol + 1) * s.rows * s.plane * 8 + 15) / 16 * 16 +
-         (size_t)2 * kb * (COLS_THREADS / 32) * 2 * 8;
+         (size_t)2 * kb * (COLS_THREADS / 32) * 2 * 16;  // 16 bytes: fixed point's two words
 }
 
 // Products per batch of the dot sums: up to 16, within COLS_RING_BYTES and
 // the CTA's shared memory.
 static int cols_batch(const ColsShape& s, bool fp32, int ncol) {
-  const size_t one = fp32 ? (size_t)ncol * s.ranks * 16 * 8 : (size_t)COLS_THREADS / 32 * 16;
+  const size_t one = fp32 ? (size_t)ncol * s.ranks * 16 * 8 : (size_t)COLS_THREADS / 32 * 32;
   int kb = 16;
   while (kb > 1 && (2 * kb * one > COLS_RING_BYTES || cols_bytes(s, fp32, ncol, kb) > COLS_MAX_SMEM))
     kb /= 2;

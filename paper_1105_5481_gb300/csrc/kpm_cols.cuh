@@ -47,6 +47,7 @@
 #pragma once
 
 #include "kpm_cols.h"
+#include "kpm_fixed.cuh"
 #include "kpm_rng.cuh"
 #include "kpm_step.cuh"
 
@@ -64,6 +65,11 @@ __device__ __forceinline__ float ldc(uint32_t a, float) {
 __device__ __forceinline__ double ldc(uint32_t a, double) {
   double v;
   asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ long long ldc(uint32_t a, long long) {
+  long long v;
+  asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
   return v;
 }
 __device__ __forceinline__ uint32_t map_addr(const void* p, uint32_t rank) {
@@ -332,6 +338,229 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
         vb[i * k.Rp + col] = w[j];
       }
   }
+}
+
+// ------------------------------------------------------------------ FP64 in fixed point
+// run_rows' task with the vectors in 64-bit fixed point (see kpm_fixed.cuh; one
+// bit less here, |v| <= 2^60 units, so that the sum of six neighbours fits 64
+// bits).  Integer sums are exact, so the uniform hopping multiplies the sum of
+// the neighbours once: 4 multiply-adds and 2 (2D) or 4 (3D) 64-bit adds for
+// the bonds of a site, where the FP64 pipe takes an FMA per bond at a 32nd of
+// that rate.  The dots' lane and warp sums are integer sums too.
+template <int DIMS, bool DS, int H, int G>
+__device__ __noinline__ void run_fixed(const ColsTask& k, int q, int C, int* err, unsigned char* smem) {
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int L = k.geom.L[DIMS - 1];
+  const int U = k.geom.stride[DIMS - 1];
+  const bool per = k.geom.periodic[DIMS - 1] != 0;
+  const int ncol = k.ncol, S = k.strips, tpc = k.tpc;
+  const int r0 = band0(L, C, q), B = band0(L, C, q + 1) - r0;
+  const int BU = k.rows * U;
+  long long* buf = reinterpret_cast<long long*>(smem);  // [2][ncol][BU]
+  const int bufn = ncol * BU;
+  Fix* dsm = reinterpret_cast<Fix*>(buf + 2 * (size_t)bufn);  // [BU] scaled diagonal (DS)
+  longlong2* ring = reinterpret_cast<longlong2*>(
+      smem + (((size_t)2 * bufn + (DS ? BU : 0)) * 8 + 15) / 16 * 16);  // [2][kb][NW][2] (hi, lo)
+  const int kb = k.batch;
+
+  const int cc = t / tpc, tt = t - cc * tpc;
+  const int strip = tt / U, u = tt - strip * U;
+  const bool have = cc < ncol && strip < S;
+  const int y0 = have ? (int)(((int64_t)B * strip) / S) : 0;
+  const int h = have ? (int)(((int64_t)B * (strip + 1)) / S) - y0 : 0;
+  const bool act = h > 0;
+  const int base = have ? cc * BU + y0 * U + u : 0;
+  const int col = k.col0 + cc;
+
+  const Fix hu = Fix::of(k.sc->hu_re), du = Fix::of(k.sc->du);
+  int of[DIMS - 1], ob[DIMS - 1];
+  bool pf[DIMS - 1], pb[DIMS - 1];  // the bond exists
+  {
+    int rem = u;
+#pragma unroll
+    for (int d = 0; d < DIMS - 1; ++d) {
+      const int Ld = k.geom.L[d], st = k.geom.stride[d];
+      const int x = rem % Ld;
+      rem /= Ld;
+      const bool p = k.geom.periodic[d] != 0;
+      of[d] = (x + 1 < Ld) ? st : (p ? -(Ld - 1) * st : 0);
+      ob[d] = (x > 0) ? -st : (p ? (Ld - 1) * st : 0);
+      pf[d] = (x + 1 < Ld) || p;
+      pb[d] = (x > 0) || p;
+    }
+  }
+  uint32_t at = 0, ab = 0;
+  bool pt = false, pe = false;
+  if (act) {
+    auto addr = [&](int y) {
+      int r = q;
+      if (y < r0 || y >= r0 + B)
+        for (r = 0; r < C - 1; ++r)
+          if (y < band0(L, C, r + 1)) break;
+      return map_addr(buf + (size_t)cc * BU + (y - band0(L, C, r)) * U + u, (uint32_t)r);
+    };
+    const int yt = r0 + y0 - 1, yb = r0 + y0 + h;
+    pt = yt >= 0 || per;
+    pe = yb < L || per;
+    if (pt) at = addr(yt >= 0 ? yt : L - 1);
+    if (pe) ab = addr(yb < L ? yb : 0);
+  }
+
+  long long x[H], w[H];
+  {
+    const unsigned long long seed = k.prm ? k.prm->seed : k.seed;
+    const unsigned long long s = (unsigned long long)(k.s + (k.prm ? k.prm->s0 : 0));
+    const Fix* src = reinterpret_cast<const Fix*>(k.ds);
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      x[j] = w[j] = 0;
+      if (j < H - G ? act : j < h) {
+        const int64_t i = (int64_t)(r0 + y0 + j) * U + u;
+        double v, im;
+        random_value<double, false>(k.n, k.R, seed, s, i, col, v, im);
+        x[j] = v < 0.0 ? -(1ll << k.fixq) : 1ll << k.fixq;
+        buf[base + j * U] = x[j];
+        if (DS && cc == 0) dsm[base + j * U] = src[i];
+      }
+    }
+  }
+  auto sync = [&]() {
+    if (C > 1) {
+      arrive();
+      wait();
+    } else {
+      __syncthreads();
+    }
+  };
+  sync();
+
+  const int nprod = k.n1;
+  const int wpc = tpc >> 5;
+  auto bulk = [&](int b, int cnt) {
+    const int items = cnt * 2 * ncol;
+    // four lanes per (product, column, dot) add the column's warps (exact sums)
+    const longlong2* rb = ring + (size_t)(b & 1) * kb * NW * 2;
+    const int sub = t & 3;
+    for (int i0 = 0; i0 < items; i0 += BT / 4) {
+      const int it = i0 + (t >> 2);
+      const bool on = it < items;
+      const int pi = it / (2 * ncol), r = it - pi * 2 * ncol, c = r >> 1, dot = r & 1;
+      long long hi = 0, lo = 0;
+      if (on)
+        for (int v = sub; v < wpc; v += 4) {
+          const longlong2 e = rb[((size_t)pi * NW + c * wpc + v) * 2 + dot];
+          hi += e.x;
+          lo += e.y;
+        }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+      }
+      if (on && sub == 0) {
+        const double unit = __longlong_as_double((long long)(1023 + 64 - 2 * k.fixq) << 52);
+        const double a = fma((double)lo, 0x1p-32, (double)hi) * unit;
+        const int step = b * kb + pi;
+        if (C == 1) k.sums[(size_t)step * 2 * k.Rp + (size_t)dot * k.Rp + k.col0 + c] = a;
+        else k.part[((size_t)q * nprod + step) * 2 * ncol + r] = a;
+      }
+    }
+  };
+
+  const uint32_t bufb = (uint32_t)((size_t)bufn * 8);
+  unsigned bad = 0;
+  int bi = 0;
+#pragma unroll 1
+  for (int m = 0; m < nprod; ++m) {
+    const int bo = bi ^ 1;
+    long long ah = 0, ac = 0, bh = 0, bc = 0;
+    if (act) {
+      const long long* X = buf + bi * bufn + base;
+      long long* Y = buf + bo * bufn + base;
+      const Fix* D = dsm + (base - cc * BU);
+      const long long xt = pt ? ldc(at + bi * bufb, 0ll) : 0;
+      const long long xb = pe ? ldc(ab + bi * bufb, 0ll) : 0;
+      constexpr int GS = H < 4 ? H : 4;
+#pragma unroll
+      for (int j0 = 0; j0 < H; j0 += GS) {
+        long long sum[GS];
+        Fix de[GS];
+#pragma unroll
+        for (int jj = 0; jj < GS; ++jj) {
+          const int j = j0 + jj;
+          sum[jj] = 0;
+          de[jj] = du;
+          if (j < H - G || j < h) {
+#pragma unroll
+            for (int d = 0; d < DIMS - 1; ++d) {
+              if (pf[d]) sum[jj] += X[j * U + of[d]];
+              if (pb[d]) sum[jj] += X[j * U + ob[d]];
+            }
+            if (DS) de[jj] = D[j * U];
+          }
+        }
+#pragma unroll
+        for (int jj = 0; jj < GS; ++jj) {
+          const int j = j0 + jj;
+          if (j < H - G || j < h) {
+            const bool last = j == H - 1 || (j + 1 >= H - G && j + 1 == h);
+            const long long s =
+                sum[jj] + (last ? xb : x[j + 1 < H ? j + 1 : j]) + (j == 0 ? xt : w[j > 0 ? j - 1 : 0]);
+            const int s0 = (int)s, s1 = (int)((s - s0) >> 32);
+            const int u0 = (int)x[j], u1 = (int)((x[j] - u0) >> 32);
+            long long a11 = mad64(hu.hi, s1, 0), a10 = mad64(hu.hi, s0, 0);
+            long long a01 = mad64(hu.lo, s1, 0), a00 = mad64(hu.lo, s0, 0);
+            if (DS || (du.hi | du.lo) != 0) {
+              a11 = mad64(de[jj].hi, u1, a11);
+              a10 = mad64(de[jj].hi, u0, a10);
+              a01 = mad64(de[jj].lo, u1, a01);
+              a00 = mad64(de[jj].lo, u0, a00);
+            }
+            const long long tt2 = a01 + (a10 >> 4) + (a00 >> 32);
+            long long v = m == 0 ? (a11 << 3) + ((tt2 + (1ll << 24)) >> 25)
+                                 : (a11 << 4) + ((tt2 + (1ll << 23)) >> 24);
+            v -= w[j];
+            bad |= (unsigned)((int)(a11 >> 32) + (1 << 25)) > (1u << 26);
+            const int v0 = (int)v, v1 = (int)((v - v0) >> 32);
+            bad |= (unsigned)(v1 + (1 << 28)) > (1u << 29);
+            Y[j * U] = v;
+            ah = mad64(u1, u1, ah);
+            bh = mad64(v1, u1, bh);
+            dot_low(ac, bc, u1, u0, v1, v0);
+            w[j] = x[j];
+            x[j] = v;
+          }
+        }
+        // at most 4 x 2^60: carried before it could overflow
+        ah += ac >> 32;
+        ac &= 0xffffffffll;
+        bh += bc >> 32;
+        bc &= 0xffffffffll;
+      }
+    }
+    if (C > 1) arrive();
+    // lanes: the upper half of the warp goes on with b, the lower with a
+    const bool up = (lane & 16) != 0;
+    long long kh = up ? bh : ah, kc = up ? bc : ac;
+    kh += __shfl_xor_sync(0xffffffffu, up ? ah : bh, 16);
+    kc += __shfl_xor_sync(0xffffffffu, up ? ac : bc, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      kh += __shfl_xor_sync(0xffffffffu, kh, o);
+      kc += __shfl_xor_sync(0xffffffffu, kc, o);
+    }
+    if ((lane & 15) == 0)
+      ring[((size_t)((m / kb) & 1) * kb + m % kb) * NW * 2 + warp * 2 + (lane >> 4)] =
+          make_longlong2(kh, kc);
+    if (C > 1) wait();
+    else __syncthreads();
+    if (m > 0 && m % kb == 0) bulk(m / kb - 1, kb);  // as in run_rows
+    bi = bo;
+  }
+  if (C > 1) __syncthreads();
+  const int bl = (nprod - 1) / kb;
+  bulk(bl, nprod - bl * kb);
+  if (bad && err) atomicOr(err, 8);
 }
 
 // ------------------------------------------------------------------ FP32, slots
@@ -730,6 +959,13 @@ __global__ void __launch_bounds__(BT, 1)
       else if (hm <= 24) run_slots<DIMS, DS, 24, 4>(k, smem);
       else if (hm <= 28) run_slots<DIMS, DS, 28, 4>(k, smem);
       else run_slots<DIMS, DS, 32, 4>(k, smem);
+    } else if (k.fixq > 0) {
+      int* err = k.prm ? const_cast<int*>(&k.prm->flags) : k.flags;
+      if (hm <= 2) run_fixed<DIMS, DS, 2, 2>(k, q, C, err, smem);
+      else if (hm <= 4) run_fixed<DIMS, DS, 4, 2>(k, q, C, err, smem);
+      else if (hm <= 8) run_fixed<DIMS, DS, 8, 4>(k, q, C, err, smem);
+      else if (hm <= 12) run_fixed<DIMS, DS, 12, 4>(k, q, C, err, smem);
+      else run_fixed<DIMS, DS, 16, 4>(k, q, C, err, smem);
     } else {
       if (hm <= 2) run_rows<DIMS, DS, 2, 2>(k, q, C, smem);
       else if (hm <= 4) run_rows<DIMS, DS, 4, 2>(k, q, C, smem);

@@ -49,6 +49,8 @@ struct ColsTask {
   int col0, ncol;
   int strips, height, tpc, rows, pitch, spi, lines;  // ColsShape
   int batch;                  // products per batch of the dot sums
+  int fixq;                   // FP64, > 0: 64-bit fixed point of unit 2^-fixq (kpm_fixed.cuh;
+                              // ds in its format, whole solves from drawn vectors)
   int n0, n1;                 // products n0 .. n1-1 (product n reads v_n, writes v_{n+1})
   int start;                  // n0 == 0: 0 draws v_0, 1 loads it from v[0]
   int keep;                   // store v_{n1-1} and v_{n1} at the end

@@ -32,6 +32,14 @@ cudaError_t launch_step_f32(bool stencil, bool cplx, StepMode mode, const StepAr
                             const LaunchCfg& cfg, cudaStream_t st);
 cudaError_t launch_step_f64(bool stencil, bool cplx, StepMode mode, const StepArgs& a,
                             const LaunchCfg& cfg, cudaStream_t st);
+// FP64 vectors of a stencil in 64-bit fixed point (kpm_fixed.cuh, a.fixq > 0):
+// the step, its CTAs per SM, and the conversions of FP64 vectors (in place, to
+// the unit 2^-q) and scaled coefficients
+cudaError_t launch_step_i64(bool stencil, bool cplx, StepMode mode, const StepArgs& a, const LaunchCfg& cfg,
+                            cudaStream_t st);
+int occ_step_i64(bool stencil, bool cplx, const StepArgs& a, int block);
+cudaError_t launch_to_fixed(int64_t count, int q, void* v, cudaStream_t st);
+cudaError_t launch_to_fix_coef(int64_t count, const void* src, void* dst, cudaStream_t st);
 // TMA-fed padded-ELL step (kpm_step_tma.cu): whether `a` admits it, its
 // launch (cfg.grid CTAs of its own size) and its CTAs per SM
 bool ell_tma_supported(const StepArgs& a, bool fp32);
@@ -138,6 +146,11 @@ cudaError_t launch_gershgorin_stencil(bool cplx, int64_t n, const StencilGeom& g
 cudaError_t launch_gershgorin_csr(bool cplx, int64_t n, const int64_t* rowptr, const int32_t* col,
                                   const double* val, double* part_min, double* part_max, int nblk,
                                   cudaStream_t st);
+// [3][nblk] partials: least and greatest on-site energy, greatest row sum of
+// the bonds' component magnitudes (g: a stencil; else a CSR's rows)
+cudaError_t launch_coef_range(bool cplx, int64_t n, const StencilGeom* g, const double* onsite,
+                              const double* hop, double t_re, double t_im, const int64_t* rowptr,
+                              const double* val, double* part, int nblk, cudaStream_t st);
 cudaError_t launch_minmax_final(const double* part_min, const double* part_max, int nblk,
                                 double* out2, cudaStream_t st);
 // Lanczos helpers (FP64; vectors are flat arrays of 2N doubles: real values
@@ -251,6 +264,14 @@ struct kpm_handle_s {
   kpm::StencilGeom geom{};
   bool has_onsite = false, has_hop = false;
   double t_re = 1.0, t_im = 0.0;
+  // Range of the coefficients (least and greatest on-site energy, greatest row
+  // sum of the bonds' components), taken when a plan first may use fixed point,
+  // and the scaled operator in the fixed-point format
+  bool ranged = false;
+  double range[3] = {0.0, 0.0, 0.0};
+  void* d_hs_fix = nullptr;
+  void* d_ds_fix = nullptr;
+  bool fix_ok = false;          // the fixed-point copies match slot 0
   double* d_onsite = nullptr;   // FP64 raw
   double* d_hop = nullptr;      // FP64 raw (masked bonds zeroed)
   // CSR
@@ -275,6 +296,7 @@ struct kpm_handle_s {
   // moments workspace
   struct Work {
     int Rp = 0, prec = -1, M = 0, nCTA = 0, block = 0;
+    bool fix_off = false;  // no memory for this plan's fixed-point operator
     bool user_v0 = false;
     void* v[2] = {nullptr, nullptr};
     size_t vbytes = 0;
@@ -313,7 +335,7 @@ struct kpm_handle_s {
     // cs.clusters > 0: the launch shape, the realisations, vectors and products
     // it was made for, the tasks with their queue, and the partials' scratch
     struct {
-      int clusters = 0, C = 0, ntasks = 0, S = 0, R = 0;
+      int clusters = 0, C = 0, ntasks = 0, S = 0, R = 0, fixq = 0;
       size_t smem = 0;
     } cs;
     void* cs_tasks = nullptr;

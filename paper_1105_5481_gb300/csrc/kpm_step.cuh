@@ -303,6 +303,34 @@ struct ChunkF32 {
   }
 };
 
+// ---------------------------------------------------------------- loads of coefficients
+template <typename T>
+struct ScalPair {
+  T x, y;
+};
+__device__ __forceinline__ float ldg_scal(const float* p, size_t i) { return __ldg(p + i); }
+__device__ __forceinline__ double ldg_scal(const double* p, size_t i) { return __ldg(p + i); }
+__device__ __forceinline__ ScalPair<float> ldg_pair(const float* p, size_t i) {
+  const float2 v = __ldg(reinterpret_cast<const float2*>(p) + i);
+  return {v.x, v.y};
+}
+__device__ __forceinline__ ScalPair<double> ldg_pair(const double* p, size_t i) {
+  const double2 v = __ldg(reinterpret_cast<const double2*>(p) + i);
+  return {v.x, v.y};
+}
+
+// The accumulator of one row's chunk (the chunk itself unless it says
+// otherwise), the chunk it ends in, and the factor of its dots.  kIssueBound:
+// instructions, not accesses in flight, limit the step.
+template <class CH, class = void>
+struct RowAcc {
+  using type = CH;
+  static constexpr bool kIssueBound = false;
+  static __device__ __forceinline__ const CH& done(const CH& acc, unsigned&) { return acc; }
+  static __device__ __forceinline__ double dot_scale(const StepArgs&) { return 1.0; }
+  static __device__ __forceinline__ void report(const StepArgs&, unsigned) {}
+};
+
 template <typename T>
 __device__ __forceinline__ void scal_from_block(const ScalarBlock* sc, T& hr, T& hi, T& du);
 template <>
@@ -322,6 +350,7 @@ __device__ __forceinline__ void scal_from_block<double>(const ScalarBlock* sc, d
 template <class CH, int DIMS, bool HAS_HOP, bool HAS_DS>
 struct StencilOp {
   using T = typename CH::T;
+  using Row = typename RowAcc<CH>::type;
   static constexpr bool CPLX = CH::CPLX;
   static constexpr bool kLines = DIMS >= 2;
   static constexpr int kDims = DIMS;
@@ -366,9 +395,9 @@ struct StencilOp {
   __device__ __forceinline__ void core(const StepArgs& a, int i, const int (&jf)[DIMS],
                                        const int (&jb)[DIMS], const bool (&hf)[DIMS],
                                        const bool (&hb)[DIMS], const T* __restrict__ Xc,
-                                       const CH& xi, CH& acc, T hu_r, T hu_i, T du,
+                                       const CH& xi, Row& acc, T hu_r, T hu_i, T du,
                                        const CH* xm = nullptr, const CH* xp = nullptr) const {
-    const T d = HAS_DS ? __ldg(reinterpret_cast<const T*>(a.ds) + i) : du;
+    const T d = HAS_DS ? ldg_scal(reinterpret_cast<const T*>(a.ds), i) : du;
     acc.axpy(d, xi);
     T fr[DIMS], fi[DIMS], br[DIMS], bi[DIMS];
 #pragma unroll
@@ -376,23 +405,34 @@ struct StencilOp {
       if constexpr (HAS_HOP) {
         const T* hs = reinterpret_cast<const T*>(a.hs);
         if constexpr (CPLX) {
-          using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
-          const T2 f = __ldg(reinterpret_cast<const T2*>(hs) + ((size_t)i * DIMS + d2));
-          const T2 bk = __ldg(reinterpret_cast<const T2*>(hs) + ((size_t)jb[d2] * DIMS + d2));
+          const ScalPair<T> f = ldg_pair(hs, (size_t)i * DIMS + d2);
+          const ScalPair<T> bk = ldg_pair(hs, (size_t)jb[d2] * DIMS + d2);
           fr[d2] = f.x;
           fi[d2] = f.y;
           br[d2] = bk.x;
           bi[d2] = -bk.y;
         } else {
-          fr[d2] = __ldg(hs + (size_t)i * DIMS + d2);
-          br[d2] = __ldg(hs + (size_t)jb[d2] * DIMS + d2);
+          fr[d2] = ldg_scal(hs, (size_t)i * DIMS + d2);
+          br[d2] = ldg_scal(hs, (size_t)jb[d2] * DIMS + d2);
           fi[d2] = bi[d2] = T(0);
         }
       } else {
         fr[d2] = hu_r; fi[d2] = hu_i; br[d2] = hu_r; bi[d2] = -hu_i;
       }
-      if (!hf[d2]) { fr[d2] = T(0); fi[d2] = T(0); }
-      if (!hb[d2]) { br[d2] = T(0); bi[d2] = T(0); }
+    }
+    // (the selects are worth a uniform branch only where issue is the limit)
+    bool edges = true;
+    if constexpr (RowAcc<CH>::kIssueBound) {
+      edges = false;
+#pragma unroll
+      for (int d2 = 0; d2 < DIMS; ++d2) edges |= a.geom.periodic[d2] == 0;
+    }
+    if (edges) {
+#pragma unroll
+      for (int d2 = 0; d2 < DIMS; ++d2) {
+        if (!hf[d2]) { fr[d2] = T(0); fi[d2] = T(0); }
+        if (!hb[d2]) { br[d2] = T(0); bi[d2] = T(0); }
+      }
     }
     const size_t rowS = (size_t)a.G * CH::SC;
     CH xf[DIMS], xb[DIMS];
@@ -426,7 +466,7 @@ struct StencilOp {
   __device__ __forceinline__ void apply_line_win(const StepArgs& a, int i, int cx,
                                                  const LineCtx& k, const T* __restrict__ Xc,
                                                  const CH& xi, const CH& xm, const CH& xp,
-                                                 CH& acc, T hu_r, T hu_i, T du) const {
+                                                 Row& acc, T hu_r, T hu_i, T du) const {
     int jf[DIMS], jb[DIMS];
     bool hf[DIMS], hb[DIMS];
     const int L0 = a.line_len;
@@ -446,7 +486,7 @@ struct StencilOp {
 
   // Row i at position cx on a line described by k (line traversal).
   __device__ __forceinline__ void apply_line(const StepArgs& a, int i, int cx, const LineCtx& k,
-                                             const T* __restrict__ Xc, const CH& xi, CH& acc,
+                                             const T* __restrict__ Xc, const CH& xi, Row& acc,
                                              T hu_r, T hu_i, T du) const {
     int jf[DIMS], jb[DIMS];
     bool hf[DIMS], hb[DIMS];
@@ -468,7 +508,7 @@ struct StencilOp {
 
   // Row i in natural order: coordinates decoded from the index.
   __device__ __forceinline__ void apply(const StepArgs& a, int64_t i64, const T* __restrict__ Xc,
-                                        const CH& xi, CH& acc, T hu_r, T hu_i, T du) const {
+                                        const CH& xi, Row& acc, T hu_r, T hu_i, T du) const {
     const int i = (int)i64;
     int jf[DIMS], jb[DIMS];
     bool hf[DIMS], hb[DIMS];
@@ -492,24 +532,25 @@ struct StencilOp {
 template <class CH>
 struct CsrOp {
   using T = typename CH::T;
+  using Row = typename RowAcc<CH>::type;
   static constexpr bool CPLX = CH::CPLX;
   static constexpr bool kLines = false;
-  static constexpr int kMinBlocks = KPM_SPARSE_MIN_BLOCKS;
+  // (an accumulator apart from the chunk takes more registers)
+  static constexpr int kMinBlocks = std::is_same<Row, CH>::value ? KPM_SPARSE_MIN_BLOCKS : 2;
   static constexpr bool kPairReduce = false;
   struct LineCtx {};
   __device__ __forceinline__ void hop(const T* V, int64_t k, T& hr, T& hi) const {
     if constexpr (CPLX) {
-      using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
-      const T2 h = __ldg(reinterpret_cast<const T2*>(V) + k);
+      const ScalPair<T> h = ldg_pair(V, (size_t)k);
       hr = h.x;
       hi = h.y;
     } else {
-      hr = __ldg(V + k);
+      hr = ldg_scal(V, (size_t)k);
       hi = T(0);
     }
   }
   __device__ __forceinline__ void apply(const StepArgs& a, int64_t i, const T* __restrict__ Xc,
-                                        const CH& xi, CH& acc, T, T, T du) const {
+                                        const CH& xi, Row& acc, T, T, T du) const {
     acc.axpy(du, xi);
     const int64_t k0 = __ldg(a.rowptr + i), k1 = __ldg(a.rowptr + i + 1);
     const T* V = reinterpret_cast<const T*>(a.vals);
@@ -547,13 +588,15 @@ struct CsrOp {
 template <class CH, int W>
 struct EllOp {
   using T = typename CH::T;
+  using Row = typename RowAcc<CH>::type;
   static constexpr bool CPLX = CH::CPLX;
   static constexpr bool kLines = false;
-  static constexpr int kMinBlocks = KPM_SPARSE_MIN_BLOCKS;
+  // (an accumulator apart from the chunk takes more registers)
+  static constexpr int kMinBlocks = std::is_same<Row, CH>::value ? KPM_SPARSE_MIN_BLOCKS : 2;
   static constexpr bool kPairReduce = false;
   struct LineCtx {};
   __device__ __forceinline__ void apply(const StepArgs& a, int64_t i, const T* __restrict__ Xc,
-                                        const CH& xi, CH& acc, T, T, T du) const {
+                                        const CH& xi, Row& acc, T, T, T du) const {
     acc.axpy(du, xi);
     const int2* cp = reinterpret_cast<const int2*>(a.col + (size_t)i * W);
     int j[W];
@@ -565,7 +608,6 @@ struct EllOp {
       j[2 * k + 1] = c2.y;
     }
     if constexpr (CPLX) {
-      using T4 = typename std::conditional<sizeof(T) == 4, float4, double4>::type;
       if constexpr (sizeof(T) == 4) {
         const float4* vp = reinterpret_cast<const float4*>(a.vals) + (size_t)i * (W / 2);
 #pragma unroll
@@ -574,19 +616,18 @@ struct EllOp {
           hr[2 * k] = v.x; hi[2 * k] = v.y; hr[2 * k + 1] = v.z; hi[2 * k + 1] = v.w;
         }
       } else {
-        const double2* vp = reinterpret_cast<const double2*>(a.vals) + (size_t)i * W;
+        const T* vp = reinterpret_cast<const T*>(a.vals);
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-          const double2 v = __ldg(vp + k);
+          const ScalPair<T> v = ldg_pair(vp, (size_t)i * W + k);
           hr[k] = v.x; hi[k] = v.y;
         }
       }
-      (void)sizeof(T4);
     } else {
       const T* vp = reinterpret_cast<const T*>(a.vals) + (size_t)i * W;
 #pragma unroll
       for (int k = 0; k < W; ++k) {
-        hr[k] = __ldg(vp + k);
+        hr[k] = ldg_scal(vp, (size_t)k);
         hi[k] = T(0);
       }
     }
@@ -607,12 +648,15 @@ struct EllOp {
 // UNROLL4: four-pass chunks that stay on one lattice line are fully unrolled,
 // the x-window rotating through registers instead of being moved (measured:
 // 5 % faster in the batched persistent kernel, 5 % slower in the single-solve
-// step, where the compiler's hoisting across passes costs more than it saves).
+// step, where the compiler's hoisting across passes costs more than it saves;
+// the fixed-point step, bound by issue, gains 5 %).
 template <class CH, int MODE, class OP, bool SWEEP = true, bool UNROLL4 = false>
 __device__ __forceinline__ void step_rows(const StepArgs& a, const OP& op, int cta, int ncta,
                                           int ycol, typename CH::Acc& s, bool first = false) {
   using T = typename CH::T;
+  using Row = typename RowAcc<CH>::type;
   constexpr int SC = CH::SC;
+  unsigned bad = 0;  // see RowAcc
   const int Gt = a.Gt;
   const int t = threadIdx.x;
   const int c = ycol * Gt + t % Gt;       // chunk within the row
@@ -651,7 +695,7 @@ __device__ __forceinline__ void step_rows(const StepArgs& a, const OP& op, int c
         const size_t rowS2 = rowS;
         auto pass = [&](int i, int cxp, const CH& xm, const CH& x0, const CH& xp) {
           const size_t base = (size_t)i * rowS2;
-          CH acc;
+          Row acc;
           if (MODE == MODE_STEP || (MODE == MODE_DYN && !first)) {
             CH wv;
             wv.ld_cs(Wc + base);
@@ -661,8 +705,9 @@ __device__ __forceinline__ void step_rows(const StepArgs& a, const OP& op, int c
           }
           op.apply_line_win(a, i, cxp, lctx, Xc, x0, xm, xp, acc, hu_r, hu_i, du);
           if (MODE == MODE_FIRST || (MODE == MODE_DYN && first)) acc.half();
-          acc.st(Yc + base);
-          if constexpr (MODE != MODE_SPMV) CH::acc_add(s, x0, acc);
+          const CH& y = RowAcc<CH>::done(acc, bad);
+          y.st(Yc + base);
+          if constexpr (MODE != MODE_SPMV) CH::acc_add(s, x0, y);
         };
         if (UNROLL4 && np == 4 && cx + 4 <= Lx && lctx.valid) {
           // four positions on one line: the window rotates through unrolled
@@ -729,7 +774,8 @@ __device__ __forceinline__ void step_rows(const StepArgs& a, const OP& op, int c
         if (i >= a.n) continue;
       }
       const size_t base = (size_t)i * rowS;
-      CH xi, acc;
+      CH xi;
+      Row acc;
       xi.ld_x(Xc + base);
       if (MODE == MODE_STEP || (MODE == MODE_DYN && !first)) {
         CH wv;
@@ -745,10 +791,12 @@ __device__ __forceinline__ void step_rows(const StepArgs& a, const OP& op, int c
         op.apply(a, i, Xc, xi, acc, hu_r, hu_i, du);
       }
       if (MODE == MODE_FIRST || (MODE == MODE_DYN && first)) acc.half();
-      acc.st(Yc + base);
-      if constexpr (MODE != MODE_SPMV) CH::acc_add(s, xi, acc);
+      const CH& y = RowAcc<CH>::done(acc, bad);
+      y.st(Yc + base);
+      if constexpr (MODE != MODE_SPMV) CH::acc_add(s, xi, y);
     }
   }
+  RowAcc<CH>::report(a, bad);
 }
 
 // CTA-wide sum of the threads' moment dots: lanes sharing a column are
@@ -836,7 +884,7 @@ __device__ __forceinline__ void cta_reduce(const StepArgs& a, typename CH::Acc s
       const int which = o / Rt, col = o % Rt, cc = col / VEC, k = col % VEC;
       double sum = 0.0;
       for (int qq = 0; qq < nq; ++qq) sum += red[((qq * Gt + cc) * 2 + which) * VEC + k];
-      dst[which * Rp + ycol * Rt + col] = sum;
+      dst[which * Rp + ycol * Rt + col] = sum * RowAcc<CH>::dot_scale(a);
     }
   }
 }
@@ -865,7 +913,7 @@ __global__ void __launch_bounds__(256, OP::kMinBlocks) cheb_step_kernel(const St
   const OP op;
   typename CH::Acc s;
   CH::acc_zero(s);
-  step_rows<CH, MODE, OP>(a, op, blockIdx.x, gridDim.x, blockIdx.y, s);
+  step_rows<CH, MODE, OP, true, RowAcc<CH>::kIssueBound>(a, op, blockIdx.x, gridDim.x, blockIdx.y, s);
   if constexpr (MODE != MODE_SPMV) {
     extern __shared__ double red[];
     cta_reduce<CH, OP::kPairReduce>(a, s, blockIdx.y, red,

@@ -6,6 +6,18 @@
 namespace kpm {
 
 template <class CH, class F>
+auto visit_stencil(const StepArgs& a, F&& f) {
+  const bool hh = a.hs != nullptr, hd = a.ds != nullptr;
+#define KPM_CASE(D, H, S) \
+  if (a.geom.dims == D && hh == H && hd == S) return f.template operator()<StencilOp<CH, D, H, S>>();
+  KPM_CASE(3, true, false) KPM_CASE(3, true, true) KPM_CASE(3, false, false) KPM_CASE(3, false, true)
+  KPM_CASE(2, true, false) KPM_CASE(2, true, true) KPM_CASE(2, false, false) KPM_CASE(2, false, true)
+  KPM_CASE(1, true, false) KPM_CASE(1, true, true) KPM_CASE(1, false, false)
+#undef KPM_CASE
+  return f.template operator()<StencilOp<CH, 1, false, true>>();
+}
+
+template <class CH, class F>
 auto visit_op(bool stencil, const StepArgs& a, F&& f) {
   if (!stencil) {
     switch (a.ell_w) {
@@ -16,14 +28,7 @@ auto visit_op(bool stencil, const StepArgs& a, F&& f) {
       default: return f.template operator()<CsrOp<CH>>();
     }
   }
-  const bool hh = a.hs != nullptr, hd = a.ds != nullptr;
-#define KPM_CASE(D, H, S) \
-  if (a.geom.dims == D && hh == H && hd == S) return f.template operator()<StencilOp<CH, D, H, S>>();
-  KPM_CASE(3, true, false) KPM_CASE(3, true, true) KPM_CASE(3, false, false) KPM_CASE(3, false, true)
-  KPM_CASE(2, true, false) KPM_CASE(2, true, true) KPM_CASE(2, false, false) KPM_CASE(2, false, true)
-  KPM_CASE(1, true, false) KPM_CASE(1, true, true) KPM_CASE(1, false, false)
-#undef KPM_CASE
-  return f.template operator()<StencilOp<CH, 1, false, true>>();
+  return visit_stencil<CH>(a, f);
 }
 
 template <class CH, int MODE>
