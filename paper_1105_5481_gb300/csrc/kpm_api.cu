@@ -717,6 +717,7 @@ kpm_status kpm_create_stencil(const kpm_stencil_desc* d, kpm_field field, kpm_ha
     h->geom.periodic[k] = k < d->dims ? (d->periodic[k] != 0) : 0;
     stride *= h->geom.L[k];
   }
+  for (int k = 0; k < 2; ++k) h->geom.by[k] = fast_div((unsigned)h->geom.L[k]);
   h->t_re = d->t_re;
   h->t_im = h->cplx ? d->t_im : 0.0;
   // stored entries: closed form for unmasked lattices, one host pass otherwise

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "kpm_fastdiv.cuh"
+
 namespace kpm {
 
 // ----------------------------------------------------------------- operator descriptions
@@ -22,6 +24,7 @@ struct StencilGeom {
   int L[3];
   int stride[3];
   int periodic[3];
+  FastDiv by[2];            // division by L[0] and L[1]
 };
 
 // Per-call parameters that live in device memory so that a captured graph

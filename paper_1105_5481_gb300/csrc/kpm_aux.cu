@@ -90,10 +90,20 @@ __global__ void rng_init_kernel(int64_t n, int Rp, const RunParams* __restrict__
   const int R = prm->R;
   const unsigned long long seed = prm->seed;
   const unsigned long long s = (unsigned long long)(prm->s + prm->s0);
-  const int64_t total = n * Rp;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x)
-    random_entry<T, CPLX>(v0, n, Rp, R, seed, s, e);
+  // Bound by instructions, not by the 8 bytes written: (i, r) advance by the
+  // grid's stride, one 64-bit division per thread instead of two per element
+  // (4.1 M sites x 32 complex FP32 columns: 0.3 ms less)
+  const int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned step = gridDim.x * blockDim.x, di = step / Rp, dr = step % Rp;
+  int64_t i = e0 / Rp;
+  int r = (int)(e0 - i * Rp);
+  for (; i < n; i += di, r += dr) {
+    if (r >= Rp) {
+      r -= Rp;
+      if (++i >= n) break;
+    }
+    random_entry<T, CPLX>(v0, n, Rp, R, seed, s, i, r);
+  }
 }
 
 template <typename T, bool CPLX>
@@ -1328,7 +1338,7 @@ cudaError_t launch_prescale_csr(bool fp32, bool cplx, int64_t nnz, const double*
 
 cudaError_t launch_rng_init(bool fp32, bool cplx, int64_t n, int Rp, const RunParams* prm, void* v0,
                             cudaStream_t st) {
-  const unsigned g = blocks_for(n * Rp, 256);
+  const unsigned g = std::min(blocks_for(n * Rp, 256), 152u * 16u);
   if (fp32) {
     if (cplx) rng_init_kernel<float, true><<<g, 256, 0, st>>>(n, Rp, prm, (float*)v0);
     else rng_init_kernel<float, false><<<g, 256, 0, st>>>(n, Rp, prm, (float*)v0);

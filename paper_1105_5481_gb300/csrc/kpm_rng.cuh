@@ -48,15 +48,16 @@ __device__ __forceinline__ void random_value(int64_t n, int R, unsigned long lon
                                      (unsigned long long)n + (unsigned long long)i;
   const unsigned long long z = draw(seed, 0, ctr);
   if (CPLX) {
-    const double u = (double)(z >> 11) * 0x1.0p-53;
     if (sizeof(T) == 8) {
+      const double u = (double)(z >> 11) * 0x1.0p-53;
       double sv, cv;
       sincospi(2.0 * u, &sv, &cv);
       re = (T)cv;
       im = (T)sv;
     } else {
       float sv, cv;
-      sincospif(2.0f * (float)u, &sv, &cv);
+      // u rounded once to FP32 (the scaling is exact), off the FP64 pipe
+      sincospif(2.0f * (__ull2float_rn(z >> 11) * 0x1.0p-53f), &sv, &cv);
       re = (T)cv;
       im = (T)sv;
     }
@@ -65,13 +66,12 @@ __device__ __forceinline__ void random_value(int64_t n, int R, unsigned long lon
   }
 }
 
-// Writes element e = i * Rp + r of the start block (zero for padded columns r >= R).
+// Writes entry (i, r) of the start block (zero for padded columns r >= R).
 template <typename T, bool CPLX>
 __device__ __forceinline__ void random_entry(T* v0, int64_t n, int Rp, int R,
                                              unsigned long long seed, unsigned long long s,
-                                             int64_t e) {
-  const int64_t i = e / Rp;
-  const int r = (int)(e % Rp);
+                                             int64_t i, int r) {
+  const int64_t e = i * Rp + r;
   int64_t ore = e, oim = e;
   if (CPLX) cplx_offsets<T>(i, r, Rp, ore, oim);
   if (r >= R) {
@@ -83,6 +83,13 @@ __device__ __forceinline__ void random_entry(T* v0, int64_t n, int Rp, int R,
   random_value<T, CPLX>(n, R, seed, s, i, r, re, im);
   v0[ore] = re;
   if (CPLX) v0[oim] = im;
+}
+// the same of element e = i * Rp + r
+template <typename T, bool CPLX>
+__device__ __forceinline__ void random_entry(T* v0, int64_t n, int Rp, int R,
+                                             unsigned long long seed, unsigned long long s,
+                                             int64_t e) {
+  random_entry<T, CPLX>(v0, n, Rp, R, seed, s, e / Rp, (int)(e % Rp));
 }
 
 }  // namespace kpm
