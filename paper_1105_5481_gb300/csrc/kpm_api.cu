@@ -979,15 +979,21 @@ kpm_status kpm_bounds(kpm_handle h, int lanczos_steps, double pad_eps, uint64_t 
       cleanup();
       return st_;
     }
-    if ((st_ = ensure_scaled(h, 2, false)) != KPM_OK) {
+    // the product is H itself: a CSR's own entries serve, a stencil needs -t
+    const bool own = !h->stencil && !h->dense;
+    if (!own && (st_ = ensure_scaled(h, 2, false)) != KPM_OK) {
       cudaStreamSynchronize(st);
       cleanup();
       return st_;
     }
-    KPM_TRY(prescale(h, 2, false, true, st));
+    if (own)
+      KPM_TRY(launch_prescale_csr(false, h->cplx, 0, h->d_val, h->d_prm, true, nullptr, h->d_sc + 2, st));
+    else
+      KPM_TRY(prescale(h, 2, false, true, st));
     int Rp, G;
     padded_width(1, false, h->cplx, &Rp, &G);
     StepArgs sa = base_args(h, 2, Rp, G);
+    if (own) sa.vals = h->ell_w > 0 ? h->d_ell_val : h->d_val;
     int block, grid;
     plan_grid(h, false, sa, &block, &grid);
     KPM_TRY(launch_lanczos_start(h->cplx, h->n, (unsigned long long)seed, Q, st));
@@ -999,7 +1005,7 @@ kpm_status kpm_bounds(kpm_handle h, int lanczos_steps, double pad_eps, uint64_t 
       KPM_TRY(launch_op(h, false, MODE_SPMV, sa, LaunchCfg{block, grid}, st));
       // three-term step against q_j, q_{j-1}, then one full Gram-Schmidt pass
       // (partial: where the step is flagged)
-      KPM_TRY(launch_lz_local_dots(h->cplx, h->n, Q, len, j, y, part_loc, nblk, st));
+      KPM_TRY(launch_lz_local_dots(h->cplx, h->n, Q, len, j, y, part_loc, nblk, partial, st));
       if (partial) {
         KPM_TRY(launch_lz_three_term(h->cplx, h->n, Q, len, j, part_loc, y, part, alpha, nblk, st));
         KPM_TRY(launch_lz_omega(j, k, nblk, part, alpha, beta, omega, flag, st));

@@ -263,7 +263,11 @@ __global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* 
 }
 
 // ------------------------------------------------------------------ Gershgorin
-__device__ __forceinline__ double cabs2(double re, double im) { return hypot(re, im); }
+__device__ __forceinline__ double cabs2(double re, double im) {
+  // (hypot's scaling, half of its FP64 instructions, only where it is needed)
+  const double m = fma(re, re, im * im);
+  return m > 1e-280 && m < 1e280 ? sqrt(m) : hypot(re, im);
+}
 
 __global__ void gershgorin_stencil_kernel(bool cplx, int64_t n, StencilGeom g,
                                           const double* __restrict__ onsite,
@@ -484,9 +488,10 @@ __device__ __forceinline__ double warp_sum(double v) {
 //                    where one may exceed the threshold the step (and the next
 //                    one) is flagged;
 //   lz_reorth_dots, dots_final, lz_update_norm: leave at once unless flagged.
-// 30 steps on a million-site complex lattice as CSR: 5.0 ms (no step flagged),
-// 12.1 ms with the pass in every step; on small vectors the launches that
-// decide would outweigh it.
+// 30 steps on a million-site complex lattice as CSR: 4.0 ms (no step flagged;
+// 54 us of a step the product, 15 + 19 the dots and the update, 11 the
+// normalisation, 20 the launches that decide or leave), 12.1 ms with the pass in
+// every step; on small vectors the launches that decide would outweigh it.
 // GB300 runs FP64 at 1/64 of its FP32 rate, so these kernels are bound by
 // FP64 instruction issue; the per-block sums of many values use a
 // recursive-halving warp reduction (about one add per value per lane instead
@@ -548,6 +553,18 @@ __device__ __forceinline__ void cdot_acc(double& re, double& im, double2 q, doub
   }
 }
 
+template <bool CPLX>
+__device__ __forceinline__ double cdot_re(double re, double2 q, double2 y) {
+  return CPLX ? fma(q.x, y.x, fma(q.y, y.y, re)) : fma(q.x, y.x, re);
+}
+
+// y -= c * q (real c)
+template <bool CPLX>
+__device__ __forceinline__ void raxpy_sub(double2& y, double c, double2 q) {
+  y.x = fma(-c, q.x, y.x);
+  if constexpr (CPLX) y.y = fma(-c, q.y, y.y);
+}
+
 // y -= c * q
 template <bool CPLX>
 __device__ __forceinline__ void caxpy_sub(double2& y, double cr, double ci, double2 q) {
@@ -559,23 +576,35 @@ __device__ __forceinline__ void caxpy_sub(double2& y, double cr, double ci, doub
   }
 }
 
-// part[blk][4] = (<q_j|y>, <q_{j-1}|y>) as (re, im, re, im); qm = NULL at j = 0
-template <bool CPLX>
+// part[blk][4] = (<q_j|y>, <q_{j-1}|y>) as (re, im, re, im); qm = NULL at j = 0.
+// RE: the real parts alone, half the FP64 work.  Both products are real but for
+// rounding (H is Hermitian; <q_{j-1}|y> = beta_{j-1}), so that what the imaginary
+// parts would remove is of the size of the rounding of y.
+template <bool CPLX, bool RE>
 __global__ void __launch_bounds__(LZ_BLOCK) lz_local_dots_kernel(int64_t n,
                                                                  const double2* __restrict__ qj,
                                                                  const double2* __restrict__ qm,
                                                                  const double2* __restrict__ y,
                                                                  double* part) {
-  __shared__ double red[LZ_WARPS * 4];
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  constexpr int V = RE ? 2 : 4;
+  __shared__ double red[LZ_WARPS * V];
+  double acc[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) acc[v] = 0.0;
   for (int64_t e = (int64_t)blockIdx.x * LZ_BLOCK + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * LZ_BLOCK) {
     const double2 yv = y[e];
-    cdot_acc<CPLX>(acc[0], acc[1], qj[e], yv);
-    if (qm) cdot_acc<CPLX>(acc[2], acc[3], qm[e], yv);
+    if constexpr (RE) {
+      acc[0] = cdot_re<CPLX>(acc[0], qj[e], yv);
+      if (qm) acc[1] = cdot_re<CPLX>(acc[1], qm[e], yv);
+    } else {
+      cdot_acc<CPLX>(acc[0], acc[1], qj[e], yv);
+      if (qm) cdot_acc<CPLX>(acc[2], acc[3], qm[e], yv);
+    }
   }
-  const double tot = block_multi_sum<4>(acc, red);
-  if (threadIdx.x < 4) part[(size_t)blockIdx.x * 4 + threadIdx.x] = tot;
+  const double tot = block_multi_sum<V>(acc, red);
+  if (threadIdx.x < V) part[(size_t)blockIdx.x * 4 + (RE ? 2 : 1) * threadIdx.x] = tot;
+  if (RE && threadIdx.x < 2) part[(size_t)blockIdx.x * 4 + 2 * threadIdx.x + 1] = 0.0;
 }
 
 // The sums over the blocks of lz_local_dots' four partials (every block in the
@@ -593,7 +622,7 @@ __device__ __forceinline__ void local_coefs(const double* __restrict__ part_loc,
   __syncthreads();
 }
 
-// y' = y - c_j q_j - c_{j-1} q_{j-1}, part[blk] = partial |y'|^2, alpha[j].
+// y' = y - c_j q_j - c_{j-1} q_{j-1} (real coefficients), part[blk] = partial |y'|^2, alpha[j].
 template <bool CPLX>
 __global__ void __launch_bounds__(LZ_BLOCK) lz_three_term_kernel(
     int64_t n, const double2* __restrict__ qj, const double2* __restrict__ qm, int j,
@@ -601,14 +630,14 @@ __global__ void __launch_bounds__(LZ_BLOCK) lz_three_term_kernel(
   __shared__ double s_c[4];
   __shared__ double red[LZ_WARPS];
   local_coefs<CPLX>(part_loc, nblk_loc, s_c);
-  const double c0r = s_c[0], c0i = CPLX ? s_c[1] : 0.0, c1r = s_c[2], c1i = CPLX ? s_c[3] : 0.0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) alpha[j] = c0r;
+  const double c0 = s_c[0], c1 = s_c[2];
+  if (blockIdx.x == 0 && threadIdx.x == 0) alpha[j] = c0;
   double acc[1] = {0.0};
   for (int64_t e = (int64_t)blockIdx.x * LZ_BLOCK + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * LZ_BLOCK) {
     double2 yv = y[e];
-    caxpy_sub<CPLX>(yv, c0r, c0i, qj[e]);
-    if (qm) caxpy_sub<CPLX>(yv, c1r, c1i, qm[e]);
+    raxpy_sub<CPLX>(yv, c0, qj[e]);
+    if (qm) raxpy_sub<CPLX>(yv, c1, qm[e]);
     y[e] = yv;
     acc[0] = fma(yv.x, yv.x, acc[0]);
     if constexpr (CPLX) acc[0] = fma(yv.y, yv.y, acc[0]);
@@ -765,6 +794,8 @@ __global__ void dots_final_kernel(const double* part, int nblk, int j, double* o
 
 // beta_j = ||y|| from the norm partials (each block sums them in the same
 // order; block 0 stores beta_j), then q_{j+1} = y / beta_j.
+// One resident wave of blocks: each sums the partial norms itself, and with a
+// block per 256 scalars those sums took 25 us of a million-site complex step (11).
 __global__ void lanczos_next_kernel(int64_t len, const double* __restrict__ y,
                                     const double* __restrict__ part, int nblk, double* beta, int j,
                                     double* qnext) {
@@ -787,31 +818,46 @@ __global__ void lanczos_next_kernel(int64_t len, const double* __restrict__ y,
 }
 
 // ------------------------------------------------------------------ tridiagonal bounds
-// Number of eigenvalues of the m x m symmetric tridiagonal T below x (Sturm count
-// from the signs of the LDL^T pivots of T - x I).
-__device__ int sturm_count(const double* al, const double* be, int m, double x) {
+// The chain of dependent FP64 operations bounds this kernel (one division takes
+// about 0.5 us): 305 us for 30 steps with a division per pivot and per component,
+// 156 with the forms below.  T is scaled by a power of two to entries of
+// order one.
+constexpr int TD_MAXM = 256;
+
+// Number of eigenvalues of the m x m symmetric tridiagonal T below x: the sign
+// changes of the leading principal minors of T - x I (Givens, 1954), from their
+// three-term recurrence.  b2: squares of the off-diagonal.  Entries are of order
+// one, so 256 steps cannot overflow; small minors are scaled up together.  A
+// vanishing minor counts as a change of sign.
+__device__ int sturm_count(const double* al, const double* b2, int m, double x) {
   int cnt = 0;
-  double d = 1.0;
-  for (int j = 0; j < m; ++j) {
-    const double b2 = j > 0 ? be[j - 1] * be[j - 1] : 0.0;
-    d = (al[j] - x) - (j > 0 ? b2 / d : 0.0);
-    if (d == 0.0) d = -1e-300;
-    if (d < 0.0) ++cnt;
+  double p0 = 1.0, p1 = al[0] - x;
+  for (int j = 1;; ++j) {
+    if (p1 == 0.0) p1 = -1e-300 * p0;
+    cnt += (__double2hiint(p0) ^ __double2hiint(p1)) < 0;
+    if (j == m) return cnt;
+    const double p2 = fma(al[j] - x, p1, -(b2[j - 1] * p0));
+    p0 = p1;
+    p1 = p2;
+    const int e = max(__double2hiint(p0) & 0x7ff00000, __double2hiint(p1) & 0x7ff00000);
+    if (e < (723 << 20)) {
+      p0 *= 0x1p300;
+      p1 *= 0x1p300;
+    }
   }
-  return cnt;
 }
 
 // k-th smallest eigenvalue (0-based), by multisection with one warp: every
 // lane evaluates the Sturm count at one of 32 interior points of the current
 // bracket, which shrinks 33-fold per round, down to adjacent doubles.  All 32
 // lanes of the calling warp must call it with the same arguments.
-__device__ double multisect_eig(const double* al, const double* be, int m, int k, double lo,
+__device__ double multisect_eig(const double* al, const double* b2, int m, int k, double lo,
                                 double hi) {
   const int lane = threadIdx.x & 31;
   for (int it = 0; it < 64; ++it) {
-    const double w = (hi - lo) / 33.0;
+    const double w = (hi - lo) * (1.0 / 33.0);
     const double x = lo + w * (double)(lane + 1);
-    const bool above = sturm_count(al, be, m, x) > k;  // eigenvalue k lies below x
+    const bool above = sturm_count(al, b2, m, x) > k;  // eigenvalue k lies below x
     const unsigned ball = __ballot_sync(0xffffffffu, above);
     const int first = ball ? __ffs(ball) - 1 : 32;      // first point above eigenvalue k
     const double nlo = first == 0 ? lo : lo + w * (double)first;
@@ -824,79 +870,102 @@ __device__ double multisect_eig(const double* al, const double* be, int m, int k
   return 0.5 * (lo + hi);
 }
 
+struct TridiagLU {  // one warp's, in shared memory
+  double dl[TD_MAXM], d[TD_MAXM], du[TD_MAXM], du2[TD_MAXM], rd[TD_MAXM], x[TD_MAXM];
+  int piv[TD_MAXM];
+};
+
 // |last component| of the normalised eigenvector of T for eigenvalue theta, by
-// two steps of inverse iteration with a tridiagonal LU with partial pivoting.
+// three steps of inverse iteration with a tridiagonal LU with partial pivoting.
+// One warp: lane 0 runs the recurrences, the lanes share the pivots' reciprocals
+// and the normalisations.
 __device__ double last_component(const double* al, const double* be, int m, double theta,
-                                 double scale) {
-  constexpr int MAXM = 256;
-  double dl[MAXM], d[MAXM], du[MAXM], du2[MAXM], x[MAXM];
-  int piv[MAXM];
+                                 double scale, TridiagLU& t) {
+  const int lane = threadIdx.x & 31;
   const double sh = theta + 1e-13 * scale;  // keep T - sh I nonsingular
-  for (int j = 0; j < m; ++j) {
-    d[j] = al[j] - sh;
-    du[j] = j + 1 < m ? be[j] : 0.0;
-    dl[j] = j + 1 < m ? be[j] : 0.0;
-    du2[j] = 0.0;
-    x[j] = 1.0;
+  for (int j = lane; j < m; j += 32) {
+    t.d[j] = al[j] - sh;
+    t.du[j] = j + 1 < m ? be[j] : 0.0;
+    t.dl[j] = j + 1 < m ? be[j] : 0.0;
+    t.du2[j] = 0.0;
+    t.x[j] = 1.0;
   }
-  // factorisation (row interchanges between j and j+1)
-  for (int j = 0; j < m - 1; ++j) {
-    if (fabs(d[j]) >= fabs(dl[j])) {
-      piv[j] = 0;
-      const double f = d[j] != 0.0 ? dl[j] / d[j] : 0.0;
-      dl[j] = f;
-      d[j + 1] -= f * du[j];
-      du2[j] = 0.0;
-    } else {
-      piv[j] = 1;
-      const double f = d[j] / dl[j];
-      d[j] = dl[j];
-      dl[j] = f;
-      const double tmp = du[j];
-      du[j] = d[j + 1];
-      d[j + 1] = tmp - f * d[j + 1];
-      if (j + 1 < m - 1) {
-        du2[j] = du[j + 1];
-        du[j + 1] = -f * du[j + 1];
-      }
-    }
-  }
-  if (d[m - 1] == 0.0) d[m - 1] = 1e-300;
-  for (int iter = 0; iter < 3; ++iter) {
-    // forward: apply L^-1 P
+  __syncwarp();
+  if (lane == 0) {
+    // factorisation (row interchanges between j and j+1)
     for (int j = 0; j < m - 1; ++j) {
-      if (piv[j] == 0) {
-        x[j + 1] -= dl[j] * x[j];
+      if (fabs(t.d[j]) >= fabs(t.dl[j])) {
+        t.piv[j] = 0;
+        const double f = t.d[j] != 0.0 ? t.dl[j] / t.d[j] : 0.0;
+        t.dl[j] = f;
+        t.d[j + 1] -= f * t.du[j];
+        t.du2[j] = 0.0;
       } else {
-        const double tmp = x[j];
-        x[j] = x[j + 1];
-        x[j + 1] = tmp - dl[j] * x[j];
+        t.piv[j] = 1;
+        const double f = t.d[j] / t.dl[j];
+        t.d[j] = t.dl[j];
+        t.dl[j] = f;
+        const double tmp = t.du[j];
+        t.du[j] = t.d[j + 1];
+        t.d[j + 1] = tmp - f * t.d[j + 1];
+        if (j + 1 < m - 1) {
+          t.du2[j] = t.du[j + 1];
+          t.du[j + 1] = -f * t.du[j + 1];
+        }
       }
     }
-    // back substitution with U (diagonal d, super du, super-super du2)
-    for (int j = m - 1; j >= 0; --j) {
-      double v = x[j];
-      if (j + 1 < m) v -= du[j] * x[j + 1];
-      if (j + 2 < m) v -= du2[j] * x[j + 2];
-      x[j] = v / (d[j] != 0.0 ? d[j] : 1e-300);
+  }
+  __syncwarp();
+  // (a pivot below the least normal number would have no finite reciprocal)
+  for (int j = lane; j < m; j += 32) t.rd[j] = 1.0 / (fabs(t.d[j]) >= 1e-300 ? t.d[j] : 1e-300);
+  __syncwarp();
+  for (int iter = 0; iter < 3; ++iter) {
+    if (lane == 0) {
+      // forward: apply L^-1 P
+      double xj = t.x[0];
+      for (int j = 0; j < m - 1; ++j) {
+        const double xn = t.x[j + 1];
+        if (t.piv[j] == 0) {
+          t.x[j] = xj;
+          xj = xn - t.dl[j] * xj;
+        } else {
+          t.x[j] = xn;
+          xj = xj - t.dl[j] * xn;
+        }
+      }
+      t.x[m - 1] = xj;
+      // back substitution with U (diagonal d, super du, super-super du2)
+      double x1 = 0.0, x2 = 0.0;
+      for (int j = m - 1; j >= 0; --j) {
+        const double v = (t.x[j] - t.du2[j] * x2) - t.du[j] * x1;
+        x2 = x1;
+        x1 = v * t.rd[j];
+        t.x[j] = x1;
+      }
     }
+    __syncwarp();
     double nrm = 0.0;
-    for (int j = 0; j < m; ++j) nrm = fmax(nrm, fabs(x[j]));
-    for (int j = 0; j < m; ++j) x[j] /= nrm;
+    for (int j = lane; j < m; j += 32) nrm = fmax(nrm, fabs(t.x[j]));
+    for (int o = 16; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
+    for (int j = lane; j < m; j += 32) t.x[j] /= nrm;
+    __syncwarp();
   }
   double n2 = 0.0;
-  for (int j = 0; j < m; ++j) n2 += x[j] * x[j];
-  return fabs(x[m - 1]) / sqrt(n2);
+  for (int j = lane; j < m; j += 32) n2 = fma(t.x[j], t.x[j], n2);
+  n2 = warp_sum(n2);
+  return fabs(t.x[m - 1]) / sqrt(n2);
 }
 
 // out = [emin, emax, a, b, theta_min, theta_max, beta_k, m].  Two warps:
-// warp 0 finds theta_min, warp 1 theta_max (multisection), lane 0 of each
-// its eigenvector's last component; thread 0 then combines.
+// warp 0 finds theta_min, warp 1 theta_max (multisection), each its eigenvector's
+// last component; thread 0 then combines.
 __global__ void tridiag_bounds_kernel(const double* alpha, const double* beta, int kmax,
                                       const double* gersh, double pad_eps, double* out) {
   __shared__ double s_theta[2], s_last[2];
   __shared__ int s_m;
-  __shared__ double s_bk, s_lo, s_hi;
+  __shared__ double s_bk, s_lo, s_hi, s_scale;
+  __shared__ double s_al[TD_MAXM], s_be[TD_MAXM], s_b2[TD_MAXM];
+  __shared__ TridiagLU s_lu[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double gmin = gersh[0], gmax = gersh[1];
   if (threadIdx.x == 0) {
@@ -916,16 +985,26 @@ __global__ void tridiag_bounds_kernel(const double* alpha, const double* beta, i
       hi = fmax(hi, alpha[j] + r);
     }
     const double span = fmax(hi - lo, 1e-300);
-    s_lo = lo - 1e-3 * span;
-    s_hi = hi + 1e-3 * span;
+    lo -= 1e-3 * span;
+    hi += 1e-3 * span;
+    s_scale = ldexp(1.0, -ilogb(fmax(fmax(fabs(lo), fabs(hi)), 1e-300)));
+    s_lo = lo * s_scale;
+    s_hi = hi * s_scale;
   }
   __syncthreads();
   const int m = s_m;
+  for (int j = threadIdx.x; j < m; j += blockDim.x) {
+    s_al[j] = alpha[j] * s_scale;
+    s_be[j] = j + 1 < m ? beta[j] * s_scale : 0.0;
+    s_b2[j] = s_be[j] * s_be[j];
+  }
+  __syncthreads();
   if (m > 0 && warp < 2) {
-    const double th = multisect_eig(alpha, beta, m, warp == 0 ? 0 : m - 1, s_lo, s_hi);
+    const double th = multisect_eig(s_al, s_b2, m, warp == 0 ? 0 : m - 1, s_lo, s_hi);
+    const double last = m > 1 ? last_component(s_al, s_be, m, th, s_hi - s_lo, s_lu[warp]) : 1.0;
     if (lane == 0) {
-      s_theta[warp] = th;
-      s_last[warp] = m > 1 ? last_component(alpha, beta, m, th, s_hi - s_lo) : 1.0;
+      s_theta[warp] = th / s_scale;
+      s_last[warp] = last;
     }
   }
   __syncthreads();
@@ -1439,13 +1518,19 @@ cudaError_t launch_lanczos_start(bool cplx, int64_t n, unsigned long long seed, 
 }
 
 cudaError_t launch_lz_local_dots(bool cplx, int64_t n, const double* Q, int64_t ldq, int j,
-                                const double* y, double* part_loc, int nblk, cudaStream_t st) {
+                                const double* y, double* part_loc, int nblk, bool real,
+                                 cudaStream_t st) {
   const double2* q = reinterpret_cast<const double2*>(Q);
   const double2* qj = q + (size_t)j * (ldq / 2);
   const double2* qm = j > 0 ? q + (size_t)(j - 1) * (ldq / 2) : nullptr;
   const double2* y2 = reinterpret_cast<const double2*>(y);
-  if (cplx) lz_local_dots_kernel<true><<<nblk, LZ_BLOCK, 0, st>>>(n, qj, qm, y2, part_loc);
-  else lz_local_dots_kernel<false><<<nblk, LZ_BLOCK, 0, st>>>(n, qj, qm, y2, part_loc);
+  if (real) {
+    if (cplx) lz_local_dots_kernel<true, true><<<nblk, LZ_BLOCK, 0, st>>>(n, qj, qm, y2, part_loc);
+    else lz_local_dots_kernel<false, true><<<nblk, LZ_BLOCK, 0, st>>>(n, qj, qm, y2, part_loc);
+  } else {
+    if (cplx) lz_local_dots_kernel<true, false><<<nblk, LZ_BLOCK, 0, st>>>(n, qj, qm, y2, part_loc);
+    else lz_local_dots_kernel<false, false><<<nblk, LZ_BLOCK, 0, st>>>(n, qj, qm, y2, part_loc);
+  }
   return counted(cudaGetLastError());
 }
 
@@ -1502,7 +1587,8 @@ cudaError_t launch_lz_omega(int j, int k, int nblk, const double* part, const do
 
 cudaError_t launch_lanczos_next(int64_t n, const double* y, const double* part, int nblk,
                                 double* beta, int j, double* qnext, cudaStream_t st) {
-  lanczos_next_kernel<<<blocks_for(2 * n, 256), 256, 0, st>>>(2 * n, y, part, nblk, beta, j, qnext);
+  lanczos_next_kernel<<<std::min(blocks_for(2 * n, 256), 152u * 8u), 256, 0, st>>>(2 * n, y, part, nblk,
+                                                                                 beta, j, qnext);
   return counted(cudaGetLastError());
 }
 

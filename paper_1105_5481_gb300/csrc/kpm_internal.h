@@ -158,7 +158,8 @@ cudaError_t launch_minmax_final(const double* part_min, const double* part_max, 
 cudaError_t launch_lanczos_start(bool cplx, int64_t n, unsigned long long seed, double* q,
                                  cudaStream_t st);
 cudaError_t launch_lz_local_dots(bool cplx, int64_t n, const double* Q, int64_t ldq, int j,
-                                const double* y, double* part_loc, int nblk, cudaStream_t st);
+                                const double* y, double* part_loc, int nblk, bool real,
+                                 cudaStream_t st);
 cudaError_t launch_lz_reorth_dots(bool cplx, int64_t n, const double* Q, int64_t ldq, int j,
                                   const double* part_loc, double* y, double* part, double* alpha,
                                   int nblk, const int* flag, cudaStream_t st);
