@@ -64,6 +64,7 @@ struct StepArgs {
   const int64_t* rowptr;  // CSR
   const int32_t* col;     // CSR column indices, or ELL [n][ell_w]
   const void* vals;       // CSR / ELL scaled values (T or complex<T>)
+  int csr_ahead;          // CSR: the form that fetches the next entries ahead
   int ell_w;              // > 0: padded ELL rows of this width (col/vals are ELL)
   // Traversal.  The rows are visited in passes of Q = (threads / Gt) rows,
   // one row per thread group.  line_len == 0: pass P covers rows P*Q .. P*Q+Q-1

@@ -533,15 +533,25 @@ struct StencilOp {
   }
 };
 
-// CSR rows: y_i = du x_i + sum_k vals[k] x_{col[k]}
-template <class CH>
+// CSR rows: y_i = du x_i + sum_k vals[k] x_{col[k]}.  Bound by the latency of the
+// chain row pointer -> columns -> gathers.  AHEAD: the columns and values of the
+// next four entries are fetched while the gathers of these four are under way, and
+// the last entries of a row go as one batch; that takes 128 registers, two CTAs per
+// SM.  Taken where those hold the grid (plan_grid).  Larger FP32 operators keep
+// three CTAs per SM: 3D 61 x 50 x 73, rows of up to 19 entries, 16 columns, 36 us per
+// product (30 ahead on a grid of two per SM, which would sum the dots in another
+// order; 44 in two waves; 39 with the dots in shared memory to make room for the
+// registers, because the L1 shrinks).
+template <class CH, bool AHEAD = false>
 struct CsrOp {
   using T = typename CH::T;
   using Row = typename RowAcc<CH>::type;
   static constexpr bool CPLX = CH::CPLX;
   static constexpr bool kLines = false;
-  // (an accumulator apart from the chunk takes more registers)
-  static constexpr int kMinBlocks = std::is_same<Row, CH>::value ? KPM_SPARSE_MIN_BLOCKS : 2;
+  // (not the FP64 pipe's form, which its arithmetic bounds, nor the batched kernel's,
+  // which has no registers for it)
+  static constexpr bool kCanAhead = CH::NC && !std::is_same<T, double>::value;
+  static constexpr int kMinBlocks = AHEAD || !std::is_same<Row, CH>::value ? 2 : KPM_SPARSE_MIN_BLOCKS;
   static constexpr bool kPairReduce = false;
   struct LineCtx {};
   __device__ __forceinline__ void hop(const T* V, int64_t k, T& hr, T& hi) const {
@@ -560,28 +570,61 @@ struct CsrOp {
     const int64_t k0 = __ldg(a.rowptr + i), k1 = __ldg(a.rowptr + i + 1);
     const T* V = reinterpret_cast<const T*>(a.vals);
     const size_t rowS = (size_t)a.G * CH::SC;
-    int64_t k = k0;
-    for (; k + 4 <= k1; k += 4) {
-      int j[4];
-      T hr[4], hi[4];
+    if constexpr (AHEAD) {
+      constexpr int B = 4;
+      const int len = (int)(k1 - k0);
+      const int32_t* col = a.col + k0;
+      int j[B];
+      T hr[B], hi[B];
+      auto fetch = [&](int k) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        j[u] = __ldg(a.col + k + u);
-        hop(V, k + u, hr[u], hi[u]);
+        for (int u = 0; u < B; ++u)
+          if (k + u < len) {
+            j[u] = __ldg(col + k + u);
+            hop(V, k0 + k + u, hr[u], hi[u]);
+          }
+      };
+      fetch(0);
+      for (int k = 0; k < len; k += B) {
+        CH xj[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (k + u < len) xj[u].ld_x(Xc + (size_t)j[u] * rowS);
+        T cr[B], ci[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+          cr[u] = hr[u];
+          ci[u] = hi[u];
+        }
+        fetch(k + B);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (k + u < len) acc.cmac(cr[u], ci[u], xj[u]);
       }
-      CH xj[4];
+    } else {
+      int64_t k = k0;
+      for (; k + 4 <= k1; k += 4) {
+        int j[4];
+        T hr[4], hi[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) xj[u].ld_x(Xc + (size_t)j[u] * rowS);
+        for (int u = 0; u < 4; ++u) {
+          j[u] = __ldg(a.col + k + u);
+          hop(V, k + u, hr[u], hi[u]);
+        }
+        CH xj[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc.cmac(hr[u], hi[u], xj[u]);
-    }
-    for (; k < k1; ++k) {
-      const int j = __ldg(a.col + k);
-      T hr, hi;
-      hop(V, k, hr, hi);
-      CH xj;
-      xj.ld_x(Xc + (size_t)j * rowS);
-      acc.cmac(hr, hi, xj);
+        for (int u = 0; u < 4; ++u) xj[u].ld_x(Xc + (size_t)j[u] * rowS);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc.cmac(hr[u], hi[u], xj[u]);
+      }
+      for (; k < k1; ++k) {
+        const int j = __ldg(a.col + k);
+        T hr, hi;
+        hop(V, k, hr, hi);
+        CH xj;
+        xj.ld_x(Xc + (size_t)j * rowS);
+        acc.cmac(hr, hi, xj);
+      }
     }
   }
 };

@@ -25,7 +25,10 @@ auto visit_op(bool stencil, const StepArgs& a, F&& f) {
       case 4: return f.template operator()<EllOp<CH, 4>>();
       case 6: return f.template operator()<EllOp<CH, 6>>();
       case 8: return f.template operator()<EllOp<CH, 8>>();
-      default: return f.template operator()<CsrOp<CH>>();
+      default:
+        if constexpr (CsrOp<CH>::kCanAhead)
+          if (a.csr_ahead) return f.template operator()<CsrOp<CH, true>>();
+        return f.template operator()<CsrOp<CH>>();
     }
   }
   return visit_stencil<CH>(a, f);
