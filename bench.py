@@ -648,9 +648,14 @@ def cubic_result(args, K):
                                         vectors_compared=1, moments_compared=M, path="fp64"),
         "fp64_path": {"value": units / (ms64 / 1e3), "unit": UNIT, "ms_per_step": ms64, "steps": 2,
                       "dtype": "f64",
-                      "roofline": {"bound": "alu", "achieved": ach64, "peak": FP64_PEAK_TFLOPS,
-                                   "unit": "TFLOP/s", "frac": ach64 / FP64_PEAK_TFLOPS,
-                                   "hbm_frac": bytes64 / (step64[0] / step64[1] / 1e3) / 1e9 / hbm,
+                      "roofline": {"bound": "hbm",
+                                   "achieved": bytes64 / (step64[0] / step64[1] / 1e3) / 1e9,
+                                   "peak": hbm, "unit": "GB/s",
+                                   "frac": bytes64 / (step64[0] / step64[1] / 1e3) / 1e9 / hbm,
+                                   "fp64_equivalent_tflops": ach64,
+                                   "fp64_pipe_peak_tflops": FP64_PEAK_TFLOPS,
+                                   "note": "vectors in 64-bit fixed point, bound by integer issue "
+                                           "(KPM_FIXED=0: on the FP64 pipe)",
                                    "launch_ms": step64[0] / step64[1]},
                       "gpu_launches": l64, "clocks": clk64},
         "gpu_launches": l32, "clocks": clk32}
@@ -1056,9 +1061,10 @@ def dense_result(args, K):
 
 
 def dense_roofline(tensor, D, R, flops_step, step_s):
-    """Roofline of the dense step.  Tensor-core form: the bf16 slice products
-    (k(k+1)/2 products of 2 D^2 Rp flops, beta and k as the library chooses
-    them) per step duration, against the measured sustained bf16 GEMM rate;
+    """Roofline of the dense step.  Tensor-core form: its exact bf16 products of
+    2 D^2 Rp flops (19 residue products up to D = 4096; k(k+1)/2 slice products
+    above, beta and k as the library chooses them) per step duration, against the
+    measured sustained bf16 GEMM rate;
     FP64-pipe form: 2 D^2 R FP64 flops against the FP64 FMA rate."""
     if not tensor:
         ach = flops_step / step_s / 1e12
@@ -1071,7 +1077,8 @@ def dense_roofline(tensor, D, R, flops_step, step_s):
     beta = max(1, min(7, (24 - lg) // 2))
     k = (54 + beta - 1) // beta
     Rp = R + (R % 2)
-    tc_flops = k * (k + 1) // 2 * 2.0 * D * D * Rp
+    products = 19 if D <= 4096 else k * (k + 1) // 2
+    tc_flops = products * 2.0 * D * D * Rp
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
             peak, kind = float(json.load(f)["bf16_tflops_sustained"]), "measured (sustained cuBLAS bf16)"
@@ -1079,8 +1086,10 @@ def dense_roofline(tensor, D, R, flops_step, step_s):
         peak, kind = 1700.0, "fallback"
     ach = tc_flops / step_s / 1e12
     return {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-            "traffic": None, "kernel": f"Ozaki split: {k * (k + 1) // 2} bf16 slice products "
-                                      f"(beta={beta}, k={k}) + slicing and FP64 epilogue",
+            "traffic": None,
+            "kernel": "19 bf16 residue products + residues and recombination" if D <= 4096 else
+                      f"Ozaki split: {products} bf16 slice products (beta={beta}, k={k}) + slicing "
+                      "and FP64 epilogue",
             "flops_per_launch": tc_flops, "launch_ms": step_s * 1e3, "peak_kind": kind}
 
 

@@ -61,7 +61,9 @@ typedef enum {
 typedef enum { KPM_REAL = 0, KPM_COMPLEX = 1 } kpm_field;
 
 typedef enum {
-  KPM_FP64 = 0,               /* vectors, products and moment sums in FP64 */
+  KPM_FP64 = 0,               /* vectors, products and moment sums in FP64, or in
+                                 64-bit fixed point of FP64's accuracy where the
+                                 operator allows it (kpm_moments) */
   KPM_FP32_VEC_FP64_MOM = 1   /* vectors stored/streamed and products in FP32;
                                  moment dot products summed in FP64 from short
                                  FP32 partial sums; bounds and DOS in FP64 */
@@ -184,7 +186,14 @@ typedef struct {
  * instead runs all M/2 products of a realisation in one launch of
  * independent clusters, one per group of columns, when the planner's
  * estimate says that is faster (the column-resident solve; KPM_COLRES=0 in
- * the environment keeps the chain).  Returns KPM_EDIVERGE (after writing
+ * the environment keeps the chain).  S > 1 FP64 realisations of a 2D or 3D
+ * stencil of uniform real hopping run as column tasks of one launch where that
+ * is estimated faster than S solves in turn.  FP64 chains and column tasks of
+ * stencil and CSR operators (up to 2^18 rows of the real field, 2^20 of the
+ * complex one) with start blocks made by the library hold the vectors in 64-bit
+ * fixed point when the scaled coefficients fit the format: the same absolute
+ * resolution, off the slow FP64 pipe; KPM_FIXED=0, read when a call plans its
+ * launches, keeps that pipe.  Returns KPM_EDIVERGE (after writing
  * the outputs) when host outputs show |mu_n^r| > 1 + 1e-6 or a non-finite
  * value, and KPM_EINVAL when R exceeds one block of vectors (more than 1024
  * chunks of 16 bytes (FP64) or 32 bytes (FP32) per row, after rounding the
@@ -337,7 +346,10 @@ kpm_status kpm_step_timing(kpm_handle h, double* ms, int* step_launches);
  * the CTAs meeting at the hardware cluster barrier between products and
  * adding their moment partials through distributed shared memory in rank
  * order.  An instance's moments therefore depend only on C and the instance,
- * not on the rest of the batch.  This is the batched form of kpm_moments for
+ * not on the rest of the batch.  2D and 3D stencils of uniform real hopping take
+ * the column-strip form instead where it fits (kpm_batch_set_columns): a few
+ * columns of an instance at a time, vectors in shared memory, with the moments
+ * of the form above at C = 4 and 4 passes per chunk.  This is the batched form of kpm_moments for
  * the paper's many-realisation workload (Sec. II-A-4: S realisations, each a
  * different Hamiltonian for disorder averages). */
 typedef struct kpm_batch_s* kpm_batch;

@@ -8,6 +8,8 @@
 // load or store per thread:
 //   FP64 path (ChunkF64): 16-byte chunks, 2 real columns or 1 complex column
 //     stored (re, im).
+//     FP64 calls whose vectors fit 64-bit fixed point take ChunkI64 instead
+//     (kpm_fixed.cuh), in the same layout.
 //   FP32 path (ChunkF32): 32-byte chunks moved with 256-bit loads/stores, 8
 //     real columns or 4 complex columns stored split as (re0..re3, im0..im3),
 //     so that the complex arithmetic runs on packed f32x2 FMAs.
