@@ -370,7 +370,11 @@ __global__ void gershgorin_csr_kernel(bool cplx, int64_t n, const int64_t* __res
 // Range of the coefficients a row's product uses, for the fixed-point step: the
 // least and greatest on-site energy (0 without), and the greatest sum of the
 // components' magnitudes over a row's bonds (CSR: over its entries), as the
-// step applies them: a periodic side of length 1 or 2 has both its bonds.
+// step applies them: a periodic side of length 1 or 2 has both its bonds.  A
+// coefficient that is not finite makes the sum infinite (a maximum would pass
+// over a NaN).
+__device__ __forceinline__ double finite_or_inf(double x) { return isfinite(x) ? x : INFINITY; }
+
 __device__ __forceinline__ void coef_range_out(double lo, double hi, double t, double* part, int nblk) {
   __shared__ double s[3][256];
   const int x = threadIdx.x;
@@ -414,7 +418,7 @@ __global__ void coef_range_stencil_kernel(bool cplx, int64_t n, StencilGeom g,
       if (x + 1 < L || per) sum += mag(i, d);
       if (x > 0 || per) sum += mag(x > 0 ? i - st : i + (int64_t)(L - 1) * st, d);
     }
-    t = fmax(t, sum);
+    t = fmax(t, isfinite(on) ? finite_or_inf(sum) : INFINITY);
   }
   coef_range_out(lo, hi, t, part, gridDim.x);
 }
@@ -427,7 +431,7 @@ __global__ void coef_range_csr_kernel(bool cplx, int64_t n, const int64_t* __res
     double sum = 0.0;
     for (int64_t k = rowptr[i]; k < rowptr[i + 1]; ++k)
       sum += cplx ? fabs(val[2 * k]) + fabs(val[2 * k + 1]) : fabs(val[k]);
-    t = fmax(t, sum);
+    t = fmax(t, finite_or_inf(sum));
   }
   coef_range_out(0.0, 0.0, t, part, gridDim.x);
 }
@@ -1210,8 +1214,8 @@ __global__ void moment_stats_kernel(const double* __restrict__ pv, int nvec, int
 // 2 M / N1 + 2 N1 FMAs per node and vector instead of M: on GB300's FP64 pipe
 // (2 per SM and clock) the direct sum for 64 vectors of 2048 moments on 4096
 // nodes is 0.85 ms of FMAs alone; kpm_stats and 16 temperatures of kpm_thermo
-// on these sizes take 0.81 ms in all with this split and the integrals spread
-// over the chip, 2.12 ms before.  Every angle is a whole multiple of pi / (2K), its
+// on these sizes take 0.42 ms in all with this split, the integrals spread
+// over the chip and the workspaces pooled, 2.12 ms before.  Every angle is a whole multiple of pi / (2K), its
 // cosine and sine read from the table at the reduced index.
 //
 // Stage 1: one thread per (n1, k'), eight vectors: D as (re, im) [r][n1][k'].

@@ -197,3 +197,27 @@ def test_an_allocation_that_fails(K, S, monkeypatch):
                 mu = K.kpm_moments(h, M, R, a, b, seed=7, S=S)
                 assert np.abs(mu - mu_o).max() <= 1e-10
     assert done > 0
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("where", ["onsite", "hop", "csr"])
+def test_coefficients_that_are_not_finite(K, where, value):
+    """They give moments that are not finite, and the error that reports them."""
+    L, n = (20, 15), 300
+    on = I.onsite_disorder(3, n, 1.0)
+    hop = np.ones((n, 2))
+    if where == "onsite":
+        on[17] = value
+    elif where == "hop":
+        hop[17, 1] = value
+    if where == "csr":
+        H = O.lattice_hamiltonian(L, onsite=on)
+        val = H.val.copy()
+        val[40] = value
+        h = K.kpm_create_csr(n, H.rowptr, H.col, val)
+    else:
+        h = K.kpm_create_stencil(2, L, onsite=on, hop=hop)
+    with h:
+        with pytest.raises(K.KPMError) as e:
+            K.kpm_moments(h, 64, 4, 5.0, 0.0, seed=1)
+    assert e.value.status == K.KPM_EDIVERGE
