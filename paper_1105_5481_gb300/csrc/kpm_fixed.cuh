@@ -13,8 +13,14 @@
 //   x = (x1 2^32 + x0) 2^-q     x0 signed 32 bits, |x1| <= 2^29
 //   h = (h1 2^28 + h0) 2^-56    h0 signed 28 bits, |h| <= 7
 //   h x: h1 x1 2^60 + h1 x0 2^28 + h0 x1 2^32 + h0 x0, each class summed exactly
-//   in 64 bits over the row's bonds (sum |h| <= 15 keeps every class below
-//   2^63; the host checks it), then one rounding to the unit.
+//   in 64 bits over the row's bonds, then one rounding to the unit.
+//
+// The sums fit: sum |h| <= 15 over a row, which the host checks, bounds h1 x1 and
+// h1 x0 by 2^63 for any number of entries.  h0 does not shrink with h (|h0| <= 2^27,
+// |x0| <= 2^31), so h0 x0 holds 31 products and h0 x1 127: stencil rows have at most
+// 13 of each per component, padded rows 17, and CSR rows of any length carry the
+// upper parts of both classes to the next one every 8 entries (Row::fold; at most 17
+// products lie between).
 //
 // Measured (3D L = 64 spin lattice, 64 complex vectors): 374 us per step against
 // 939 on the FP64 pipe.  Bound by issue at 16 warps per SM (math-pipe throttle
@@ -175,6 +181,16 @@ struct ChunkI64 {
       a01[q] = mad64(h.lo, u1, a01[q]);
       a00[q] = mad64(h.lo, u0, a00[q]);
     }
+    // carries of h0 x0 (weight 1) into h0 x1 (2^32), and of that into h1 x1 (2^60)
+    __device__ __forceinline__ void fold() {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        a01[q] += a00[q] >> 32;
+        a00[q] &= 0xffffffffll;
+        a11[q] += a01[q] >> 28;
+        a01[q] &= 0xfffffffll;
+      }
+    }
     // the diagonal (often zero: no on-site terms and symmetric bounds)
     __device__ __forceinline__ void axpy(const Fix& d, const ChunkI64& x) {
       if ((d.hi | d.lo) == 0) return;
@@ -197,13 +213,14 @@ struct RowAcc<ChunkI64<CPLX>> {
   using CH = ChunkI64<CPLX>;
   using type = typename CH::Row;
   static constexpr bool kIssueBound = true;
+  static __device__ __forceinline__ void fold(type& r) { r.fold(); }
   // The sums rounded to the unit, less v_{n-1}.  `bad` is set when a value
   // leaves +-2^61: |a11| bounds the sum before its shift can overflow.
   static __device__ __forceinline__ CH done(const type& r, unsigned& bad) {
     CH y;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      // in units of 2^32 (2^-24 of the result's)
+      // in units of 2^32 (2^-24 of the result's); folded or not, the same result
       const long long t = r.a01[q] + (r.a10[q] >> 4) + (r.a00[q] >> 32);
       long long v;
       if (r.sh == 24) v = (r.a11[q] << 4) + ((t + (1ll << 23)) >> 24);

@@ -322,12 +322,14 @@ __device__ __forceinline__ ScalPair<double> ldg_pair(const double* p, size_t i) 
 }
 
 // The accumulator of one row's chunk (the chunk itself unless it says
-// otherwise), the chunk it ends in, and the factor of its dots.  kIssueBound:
-// instructions, not accesses in flight, limit the step.
+// otherwise), the chunk it ends in, and the factor of its dots.  fold is called
+// at least once per 8 entries of a CSR row.  kIssueBound: instructions, not
+// accesses in flight, limit the step.
 template <class CH, class = void>
 struct RowAcc {
   using type = CH;
   static constexpr bool kIssueBound = false;
+  static __device__ __forceinline__ void fold(CH&) {}
   static __device__ __forceinline__ const CH& done(const CH& acc, unsigned&) { return acc; }
   static __device__ __forceinline__ double dot_scale(const StepArgs&) { return 1.0; }
   static __device__ __forceinline__ void report(const StepArgs&, unsigned) {}
@@ -602,6 +604,7 @@ struct CsrOp {
 #pragma unroll
         for (int u = 0; u < B; ++u)
           if (k + u < len) acc.cmac(cr[u], ci[u], xj[u]);
+        if (k & 4) RowAcc<CH>::fold(acc);
       }
     } else {
       int64_t k = k0;
@@ -618,6 +621,7 @@ struct CsrOp {
         for (int u = 0; u < 4; ++u) xj[u].ld_x(Xc + (size_t)j[u] * rowS);
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc.cmac(hr[u], hi[u], xj[u]);
+        if ((k - k0) & 4) RowAcc<CH>::fold(acc);
       }
       for (; k < k1; ++k) {
         const int j = __ldg(a.col + k);
