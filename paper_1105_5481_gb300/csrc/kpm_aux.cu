@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* 
 
 // ------------------------------------------------------------------ Gershgorin
 __device__ __forceinline__ double cabs2(double re, double im) {
+  if (im == 0.0) return fabs(re);
   // (hypot's scaling, half of its FP64 instructions, only where it is needed)
   const double m = fma(re, re, im * im);
   return m > 1e-280 && m < 1e280 ? sqrt(m) : hypot(re, im);
@@ -1031,6 +1032,17 @@ __global__ void tridiag_bounds_kernel(const double* alpha, const double* beta, i
   out[7] = (double)m;
 }
 
+// The same without a Lanczos run: the Gershgorin enclosure alone, without the
+// shared memory and the barriers of the tridiagonal problem.
+__global__ void gershgorin_bounds_kernel(const double* gersh, double pad_eps, double* out) {
+  const double emin = gersh[0], emax = gersh[1];
+  out[0] = out[4] = emin;
+  out[1] = out[5] = emax;
+  out[2] = (emax - emin) / (2.0 - pad_eps);
+  out[3] = 0.5 * (emax + emin);
+  out[6] = out[7] = 0.0;
+}
+
 // ------------------------------------------------------------------ DOS (Eq. (fKPM))
 // coef[n] = c_n g_n mu_n with c_0 = 1, c_n = 2; Jackson g_n from the closed form.
 // Damping factor g_n of the kernel: Jackson (review Eq. 71), Lorentz
@@ -1599,6 +1611,10 @@ cudaError_t launch_lanczos_next(int64_t n, const double* y, const double* part, 
 cudaError_t launch_tridiag_bounds(const double* alpha, const double* beta, int m,
                                   const double* gersh, double pad_eps, double* out,
                                   cudaStream_t st) {
+  if (m == 0) {
+    gershgorin_bounds_kernel<<<1, 1, 0, st>>>(gersh, pad_eps, out);
+    return counted(cudaGetLastError());
+  }
   tridiag_bounds_kernel<<<1, 64, 0, st>>>(alpha, beta, m, gersh, pad_eps, out);
   return counted(cudaGetLastError());
 }
