@@ -347,9 +347,12 @@ kpm_status kpm_step_timing(kpm_handle h, double* ms, int* step_launches);
  * adding their moment partials through distributed shared memory in rank
  * order.  An instance's moments therefore depend only on C and the instance,
  * not on the rest of the batch.  2D and 3D stencils of uniform real hopping take
- * the column-strip form instead where it fits (kpm_batch_set_columns): a few
- * columns of an instance at a time, vectors in shared memory, with the moments
- * of the form above at C = 4 and 4 passes per chunk.  This is the batched form of kpm_moments for
+ * the column-strip form instead (kpm_batch_set_columns) where it fits and is
+ * estimated faster for this batch: a few columns of an instance at a time,
+ * vectors in shared memory.  With FP32 vectors its moments are those of the form
+ * above at C = 4 and 4 passes per chunk; with FP64 vectors the dots are summed in
+ * another order, of its own cluster size, which like the form is chosen for the
+ * whole batch (kpm_batch_info, kpm_batch_get_columns).  This is the batched form of kpm_moments for
  * the paper's many-realisation workload (Sec. II-A-4: S realisations, each a
  * different Hamiltonian for disorder averages). */
 typedef struct kpm_batch_s* kpm_batch;
@@ -462,7 +465,8 @@ kpm_status kpm_batch_set_staged(kpm_batch b, int staged);
  * the current traversal chunk (any output may be NULL). */
 kpm_status kpm_batch_get_staged(kpm_batch b, int* staged, int* tile_rows, int* stages);
 
-/* Column-strip form (columns = 1; what a batch starts with where it applies):
+/* Column-strip form (columns = 1; what a batch starts with where it is
+ * estimated faster than the global-memory form):
  * the instances' vector columns as independent tasks of one persistent
  * launch, each task running all products (Eq. (rn)) of a few columns of one
  * instance with v_n in the shared memory of a CTA, or of a cluster of CTAs

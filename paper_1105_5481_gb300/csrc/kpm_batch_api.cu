@@ -11,7 +11,9 @@
 #include <sys/stat.h>
 
 #include <algorithm>
+#include <functional>
 #include <numeric>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -281,6 +283,79 @@ int cols_cluster(const kpm_batch_s* b) {
     }
   }
   return best;
+}
+
+// Time of `items` (longest first) on m workers that take the next when free.
+double makespan(std::vector<double> items, int m) {
+  std::sort(items.begin(), items.end(), std::greater<double>());
+  std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
+  double end = 0.0;
+  for (double us : items) {
+    if ((int)busy.size() >= m) {
+      us += busy.top();
+      busy.pop();
+    }
+    busy.push(us);
+    end = std::max(end, us);
+  }
+  return end;
+}
+
+// Whether a batch starts with the column strips: their estimated time against the
+// global-memory form's with its defaults.  Many instances of some 1,000 to 4,000
+// sites with many vectors give the global-memory form enough CTAs to hide its round
+// trips, and the strips' second sweep for the dots then costs more than it saves:
+// 256 lattices of 32 x 32 with 32 vectors 2.06 ms (strips) against 1.66, of 16^3 7.64
+// against 5.09; 113 of 31 to 41 a side 3.72 against 3.51.  The estimates (microseconds per product, fitted
+// to 570 batches of 1 to 256 lattices of 6 to 128 (2D) or 4 to 24 (3D) a side with 4
+// to 32 FP32 vectors) are within 10 % (strips) and 15 % (global; lower by up to half
+// for power-of-two planes) of the measured times.  With 15 % to spare the strips are
+// taken in one of those batches where they are slower, by 5 %, and left in 13 where
+// they are faster, by 5 to 9 % in most.  FP64: both are bound by the FP64 pipe; its
+// instructions are counted.
+bool cols_faster(kpm_batch_s* b, int C) {
+  ColsPlan p;
+  if (!plan_cols(b, C, &p)) return false;
+  const int dims = b->handles[0]->geom.dims;
+  const bool d3 = dims == 3;
+  const int nglob = max_clusters(b, BatchConfig{});
+  if (nglob < 1) return true;
+  const int sms = b->handles[0]->num_sms, live = std::min(b->count, nglob);
+  const bool shared = live * BatchConfig{}.C > sms;  // two CTAs to an SM
+  std::vector<double> strips, global;
+  for (int i = 0; i < b->count; ++i) {
+    StepArgs a = b->inst_tasks[i].a;
+    a.Gt = a.G;
+    plan_instance(a, b->handles[i], BatchConfig{}.chunk);
+    const int64_t per_cta = ((a.passes + 3) / 4 + 3) / 4;  // chunks of four passes, four CTAs
+    const double P = (double)(std::min<int64_t>(a.passes, 4) + 4 * (per_cta - 1));
+    double us;
+    if (b->fp32) {
+      us = d3 ? 1.5 + 0.85 * P : 1.3 + 0.65 * P;
+      if (shared) us += d3 ? 1.7 + 0.15 * P : 1.9 + 0.07 * P;
+      // the vector blocks in use at a time, of this instance's size (they run in the
+      // order of their work), past half of the L2
+      us += (d3 ? 0.38 : 0.30) * P * std::max(0.0, 8.0 * a.n * a.Rp * live / 60e6 - 1.0);
+    } else {
+      // 2 (2 dims + 3) FP64 instructions of 16 clocks per warp and row, 8 warps
+      us = 4.0 + (shared ? 2.0 : 1.0) * P * 8 * 2 * (2 * dims + 3) * 16 / 1900.0;
+    }
+    global.push_back(us * (b->inst_tasks[i].M / 2));
+  }
+  const double t_global = 140.0 + makespan(global, nglob);
+  if (!b->fp32) return 1.25 * (40.0 + 1.2 * p.us) <= t_global;
+  for (const ColsTask& t : p.tasks) {
+    const int64_t passes = t.lines > 0 ? (int64_t)(t.lines + t.spi - 1) / t.spi * t.geom.L[0]
+                                       : (t.n + t.spi - 1) / t.spi;
+    const int64_t chains = std::min<int64_t>(4, (passes + 3) / 4) * t.spi;
+    const double sweeps = (double)((t.ncol * chains + COLS_THREADS - 1) / COLS_THREADS);
+    const double rows = 4.0 * ((passes + 15) / 16);  // of a chain
+    const double sites = t.ncol * (t.tpc / 32) * t.height / 16.0;  // a scheduler's, in fours
+    const double us = d3 ? 0.26 + 0.029 * t.height + 0.084 * sites + sweeps * (0.44 + 0.018 * rows)
+                         : 0.22 + 0.017 * t.height + 0.071 * sites + sweeps * (0.49 + 0.011 * rows);
+    strips.push_back(us * t.n1);
+  }
+  return 1.15 * (20.0 + makespan(strips, p.clusters)) <= t_global;
 }
 
 int cfg_clusters(kpm_batch_s* b, const BatchConfig& c) {
@@ -665,10 +740,10 @@ kpm_status kpm_batch_create(int count, const kpm_handle* handles, const kpm_para
   });
   b->inst_tasks = tasks;
   b->proto = tasks[b->order[0]].a;
-  // the column strips where they fit: a batch product of the other forms is a
-  // chain of L2 round trips (the 256-instance 2D batch: 38 ms), this one stays
-  // on its SM
-  if (const int C = cols_cluster(b)) {
+  // the column strips where they fit and are estimated faster: a batch product of
+  // the other forms is a chain of L2 round trips (the 256-instance 2D batch: 38 ms
+  // against 26), this one stays on its SM
+  if (const int C = cols_cluster(b); C && cols_faster(b, C)) {
     b->cfg.res = FORM_COLS;
     b->cfg.C = C;
   }
