@@ -224,14 +224,17 @@ bool setup_dense_tc(kpm_handle_s* h, int Rp) {
   return ok;
 }
 
+void free_cols(kpm_handle_s::Work::ColsSolve& c) {
+  dfree(c.tasks);
+  dfree(c.queue);
+  dfree(c.part);
+  c = {};
+}
+
 void free_cols(kpm_handle_s::Work& w) {
-  dfree(w.cs_tasks);
-  dfree(w.cs_queue);
-  dfree(w.cs_part);
-  w.cs_tasks = nullptr;
-  w.cs_queue = nullptr;
-  w.cs_part = nullptr;
-  w.cs = {};
+  for (auto& c : w.cs) free_cols(c);
+  w.cs_next = 0;
+  w.cs_now = -1;
 }
 
 void free_work(kpm_handle_s* h) {
@@ -706,7 +709,7 @@ kpm_status kpm_testing_last_step_form(kpm_handle h, int* form) {
   const auto& w = h->work;
   if (w.M == 0) return fail(KPM_ENOTREADY, "no kpm_moments call has planned its launches yet");
   if (h->dense) *form = w.dtc ? 3 : 2;
-  else if (w.cs.clusters > 0) *form = 6;
+  else if (w.cs_now >= 0) *form = 6;
   else if (w.cr.C > 0) *form = 5;
   else *form = w.proto.tma_stages > 0 ? (h->stencil ? 4 : 1) : 0;
   return KPM_OK;
@@ -931,7 +934,8 @@ kpm_status kpm_step_timing(kpm_handle h, double* ms, int* step_launches) {
   KPM_CUDA(cudaSetDevice(h->device));
   float t = 0.f;
   KPM_CUDA(cudaEventElapsedTime(&t, h->work.ev[0], h->work.ev[1]));
-  if (ms) *ms = h->work.cs.clusters > 0 ? t / h->work.cs.S : t;  // one launch for all realisations
+  const auto& w = h->work;
+  if (ms) *ms = w.cs_now >= 0 ? t / w.cs[w.cs_now].S : t;  // one launch for all realisations
   if (step_launches) *step_launches = h->work.M / 2;
   return KPM_OK;
 }
@@ -1153,12 +1157,13 @@ kpm_status ensure_fixed(kpm_handle_s* h) {
   if (fixed_entries(h) > 0 && !h->d_hs_fix) {
     if ((st = dalloc(&ph, (size_t)fixed_entries(h) * 8)) != KPM_OK) return st;
     h->d_hs_fix = ph;
+    h->fix_ok = false;
   }
   if (h->has_onsite && !h->d_ds_fix) {
     if ((st = dalloc(&pd, (size_t)h->n * 8)) != KPM_OK) return st;
     h->d_ds_fix = pd;
+    h->fix_ok = false;
   }
-  h->fix_ok = false;
   return KPM_OK;
 }
 
@@ -1174,12 +1179,15 @@ bool cols_solve_kind(const kpm_handle_s* h, bool fp32) {
   return !fp32 && h->stencil && !h->cplx && !h->has_hop && (h->geom.dims == 2 || h->geom.dims == 3);
 }
 
-// Plans the launch for the current buffers; leaves w.cs.clusters 0 where the
-// form does not apply.
-kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps, int fixq) {
+// Plans the launch for the current buffers into `cs`; leaves its clusters 0 where
+// the form does not apply.
+kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps, int fixq,
+                           kpm_handle_s::Work::ColsSolve& cs, cudaStream_t st) {
   auto& w = h->work;
-  free_cols(w);
-  if (S < 2 || !cols_solve_kind(h, false) || getenv("KPM_COLRES")) return KPM_OK;
+  cs.S = S;
+  cs.R = R;
+  cs.fixq = fixq;
+  if (getenv("KPM_COLRES")) return KPM_OK;
   const int dims = h->geom.dims;
   const bool ds = h->has_onsite;
   struct Try {
@@ -1222,7 +1230,8 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps, int fixq) {
       t.geom = a.geom;
       t.n = a.n;
       t.sc = a.sc;
-      t.ds = fixq > 0 && h->has_onsite ? h->d_ds_fix : a.ds;
+      // (not the step chain's, which may be in fixed point where these are not)
+      t.ds = !h->has_onsite ? nullptr : fixq > 0 ? h->d_ds_fix : h->d_ds[0];
       t.fixq = fixq;
       t.sums = w.sums + (size_t)s * steps * 2 * w.Rp;
       t.prm = h->d_prm;
@@ -1237,25 +1246,57 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps, int fixq) {
       }
       tasks.push_back(t);
     }
-  kpm_status sa = dalloc((char**)&w.cs_tasks, tasks.size() * sizeof(ColsTask));
-  if (sa == KPM_OK) sa = dalloc(&w.cs_queue, (size_t)1);
-  if (sa == KPM_OK && part) sa = dalloc(&w.cs_part, part);
+  kpm_status sa = dalloc((char**)&cs.tasks, tasks.size() * sizeof(ColsTask));
+  if (sa == KPM_OK) sa = dalloc(&cs.queue, (size_t)1);
+  if (sa == KPM_OK && part) sa = dalloc(&cs.part, part);
   if (sa != KPM_OK) {
-    free_cols(w);
-    if (sa == KPM_ENOMEM) return KPM_OK;  // the solves in turn need none of it
-    return sa;
+    free_cols(cs);
+    // the solves in turn need none of it (a later call tries again)
+    return sa == KPM_ENOMEM ? KPM_OK : sa;
   }
   for (ColsTask& t : tasks)
-    t.part = C > 1 ? (double*)((char*)w.cs_part + (size_t)t.part) : nullptr;
-  KPM_CUDA(cudaMemcpy(w.cs_tasks, tasks.data(), tasks.size() * sizeof(ColsTask),
-                      cudaMemcpyHostToDevice));
-  w.cs.C = C;
-  w.cs.fixq = fixq;
-  w.cs.ntasks = ntasks;
-  w.cs.smem = best.smem;
-  w.cs.S = S;
-  w.cs.R = R;
-  w.cs.clusters = std::min(best.clusters, ntasks);
+    t.part = C > 1 ? (double*)((char*)cs.part + (size_t)t.part) : nullptr;
+  KPM_CUDA(cudaMemcpyAsync(cs.tasks, tasks.data(), tasks.size() * sizeof(ColsTask),
+                           cudaMemcpyHostToDevice, st));
+  cs.C = C;
+  cs.ntasks = ntasks;
+  cs.smem = best.smem;
+  cs.clusters = std::min(best.clusters, ntasks);
+  return KPM_OK;
+}
+
+// The launch of S > 1 realisations in the current buffers: w.cs_now, kept or
+// planned now (-1: the solves in turn).  It stands beside the step chain's plan, so
+// that calls which alternate S, or R within one padded width, replace neither (4
+// vectors, M = 64: S = 16 and 1 in turn on 24 x 25 x 26 sites 2.77 ms a pair, 3.14
+// when each call planned anew; R = 4 and 3 in turn on 150 x 150 393 us against 453).
+kpm_status cols_solve(kpm_handle_s* h, const kpm_params* p, int R, int S, int steps, bool fix_kind,
+                      cudaStream_t st) {
+  auto& w = h->work;
+  w.cs_now = -1;
+  if (S < 2 || !cols_solve_kind(h, p->precision != KPM_FP64)) return KPM_OK;
+  auto unit = [&] {
+    return fix_kind && !w.fix_off && h->ranged ? cols_unit(fixed_unit(h, p->a, p->b)) : 0;
+  };
+  int k = 0;
+  while (k < w.COLS_PLANS && !(w.cs[k].S == S && w.cs[k].R == R)) ++k;
+  if (k == w.COLS_PLANS || (fix_kind && !w.fix_off && !h->ranged) || w.cs[k].fixq != unit()) {
+    if (k == w.COLS_PLANS) {
+      k = w.cs_next;
+      w.cs_next = (k + 1) % w.COLS_PLANS;
+    }
+    if (w.cs[k].tasks) KPM_CUDA(cudaDeviceSynchronize());  // a launch may still be reading them
+    free_cols(w.cs[k]);
+    kpm_status sa = fix_kind && !w.fix_off ? ensure_range(h) : KPM_OK;
+    if (sa == KPM_OK && unit() > 0) sa = ensure_fixed(h);
+    if (sa == KPM_ENOMEM) {  // without memory for the operator's second copy: the FP64 pipe
+      w.fix_off = true;
+      sa = KPM_OK;
+    }
+    if (sa == KPM_OK) sa = plan_cols_solve(h, R, S, steps, unit(), w.cs[k], st);
+    if (sa != KPM_OK) return sa;
+  }
+  if (w.cs[k].clusters > 0) w.cs_now = k;
   return KPM_OK;
 }
 
@@ -1327,10 +1368,8 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
   const bool rebuild = w.Rp != Rp || w.prec != p->precision || w.M != M ||
                        w.user_v0 != user_v0 || !w.ready || w.sums_bytes < sums_bytes ||
                        (w.cr.C > 0 && w.cr_R != R) ||
-                       (cols_solve_kind(h, fp32) && (w.plan_S != S || w.cr_R != R)) ||
-                       (!h->dense && w.cr.C == 0 && w.cs.clusters == 0 &&
-                        (w.proto.fixq > 0) != (h->ranged ? unit_now > 0 && !w.fix_off : fix_kind && w.proto.fixq > 0)) ||
-                       (w.cs.clusters > 0 && w.cs.fixq != (w.fix_off ? 0 : cols_unit(unit_now)));
+                       (!h->dense && w.cr.C == 0 &&
+                        (w.proto.fixq > 0) != (h->ranged ? unit_now > 0 && !w.fix_off : fix_kind && w.proto.fixq > 0));
   // The kernel sequence of one realisation.  The first call of a shape
   // launches it directly on the caller's stream (the solve is GPU-bound, so
   // the launches hide behind it); a second call of the same shape captures it
@@ -1445,25 +1484,8 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     if (dense_tc_wanted(h, fp32)) setup_dense_tc(h, Rp);
     else free_dense_tc(w);
     w.Rp = Rp;
-    if (fp32) {
-      free_cols(w);
-    } else {
-      int q = 0;
-      kpm_status sa = KPM_OK;
-      if (S > 1 && fix_kind && cols_solve_kind(h, fp32)) {
-        sa = ensure_range(h);
-        if (sa == KPM_OK && (q = cols_unit(fixed_unit(h, p->a, p->b))) > 0) sa = ensure_fixed(h);
-        if (sa == KPM_ENOMEM) {
-          w.fix_off = true;
-          q = 0;
-          sa = KPM_OK;
-        }
-      }
-      if (sa == KPM_OK) sa = plan_cols_solve(h, R, S, steps, q);
-      if (sa != KPM_OK) return sa;
-    }
-    w.plan_S = S;
-    if (fix_kind && !w.fix_off && w.cr.C == 0 && w.cs.clusters == 0) {
+    free_cols(w);
+    if (fix_kind && w.cr.C == 0) {
       // (without memory for the operator's second copy: the FP64 pipe)
       kpm_status sa = ensure_range(h);
       const int q = sa == KPM_OK ? fixed_unit(h, p->a, p->b) : 0;
@@ -1496,6 +1518,8 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     w.ready = true;
     w.direct_done = false;
   }
+  s_ = cols_solve(h, p, R, S, steps, fix_kind, st);
+  if (s_ != KPM_OK) return s_;
   if (w.out_bytes < out_bytes) {
     KPM_CUDA(cudaStreamSynchronize(st));
     dfree(w.per_vec);
@@ -1535,7 +1559,7 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     h->scaled_b[slot] = p->b;
     h->scaled_st[slot] = stream;
   }
-  if ((w.proto.fixq > 0 || (w.cs.clusters > 0 && w.cs.fixq > 0)) && !h->fix_ok) {
+  if ((w.cs_now >= 0 ? w.cs[w.cs_now].fixq : w.proto.fixq) > 0 && !h->fix_ok) {
     if (const int64_t m = fixed_entries(h))
       KPM_CUDA(launch_to_fix_coef(m, h->stencil ? h->d_hs[0] : h->d_vals[0], h->d_hs_fix, st));
     if (h->has_onsite) KPM_CUDA(launch_to_fix_coef(h->n, h->d_ds[0], h->d_ds_fix, st));
@@ -1584,12 +1608,13 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     }
     KPM_CUDA(launch_load_v0(fp32, h->cplx, h->n, R, Rp, src, w.v[0], st));
   }
-  if (w.cs.clusters > 0) {
+  if (w.cs_now >= 0) {
     // all realisations in one launch
-    KPM_CUDA(cudaMemsetAsync(w.cs_queue, 0, sizeof(int), st));
+    const auto& c = w.cs[w.cs_now];
+    KPM_CUDA(cudaMemsetAsync(c.queue, 0, sizeof(int), st));
     KPM_CUDA(cudaEventRecord(w.ev[0], st));
-    KPM_CUDA(launch_cols(false, h->geom.dims, h->has_onsite, (const ColsTask*)w.cs_tasks,
-                         w.cs.ntasks, w.cs_queue, w.cs.clusters, w.cs.C, w.cs.smem, st));
+    KPM_CUDA(launch_cols(false, h->geom.dims, h->has_onsite, (const ColsTask*)c.tasks, c.ntasks,
+                         c.queue, c.clusters, c.C, c.smem, st));
     KPM_CUDA(cudaEventRecord(w.ev[1], st));
   } else if (!w.exec && w.direct_done) {
     // second call of this shape: capture the sequence once
@@ -1609,7 +1634,7 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
       return cuda_fail(e, "capture of the moment graph");
     }
   }
-  for (int s = 0; s < S && w.cs.clusters == 0; ++s) {
+  for (int s = 0; s < S && w.cs_now < 0; ++s) {
     if (w.exec) {
       KPM_CUDA(cudaGraphLaunch(w.exec, st));
       g_launches.fetch_add(w.kernels_per_replay);
@@ -1617,7 +1642,7 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
       KPM_CUDA(enqueue(st, false));
     }
   }
-  w.direct_done = true;
+  w.direct_done |= w.cs_now < 0;
   w.timed = true;
   if (S == 1) {
     // v_{M/2-1} and v_{M/2} stay in v[] with the per-step sums: kpm_moments_extend

@@ -329,19 +329,23 @@ struct kpm_handle_s {
     // of its CTA partials
     kpm::ColresPlan cr{};
     int cr_R = 0;
-    int plan_S = 0;  // realisations the plan was made for
     double* cr_gp = nullptr;
     size_t cr_gp_doubles = 0;
-    // all S > 1 realisations as column tasks of one launch (kpm_cols.h) when
-    // cs.clusters > 0: the launch shape, the realisations, vectors and products
-    // it was made for, the tasks with their queue, and the partials' scratch
-    struct {
-      int clusters = 0, C = 0, ntasks = 0, S = 0, R = 0, fixq = 0;
+    // S > 1 realisations as column tasks of one launch (kpm_cols.h): the launch
+    // shapes of the last few (S, R) with their tasks, queue and partials' scratch,
+    // beside the plan of the step chain and dropped with it (clusters == 0: the
+    // solves in turn).  cs_now: the one the last call took, -1 for none.
+    struct ColsSolve {
+      int S = 0, R = 0, fixq = 0;
+      int clusters = 0, C = 0, ntasks = 0;
       size_t smem = 0;
-    } cs;
-    void* cs_tasks = nullptr;
-    int* cs_queue = nullptr;
-    double* cs_part = nullptr;
+      void* tasks = nullptr;
+      int* queue = nullptr;
+      double* part = nullptr;
+    };
+    static constexpr int COLS_PLANS = 4;
+    ColsSolve cs[COLS_PLANS];
+    int cs_next = 0, cs_now = -1;  // cs_next: the entry planned longest ago
     cudaEvent_t ev[2] = {nullptr, nullptr};  // recorded around the step chain in the graph
     bool timed = false;
   } work;

@@ -1,0 +1,67 @@
+"""Plans that stand beside each other: calls that alternate the realisations S, or
+the vectors R within one padded width, replace none of them (nothing is allocated
+when a shape comes again) and keep their bits; the column tasks of an operator too
+large for their fixed-point unit run beside a step chain in fixed point."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1105_5481_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def K(gpu_lib):
+    from paper_1105_5481_gb300 import kpm
+
+    return kpm
+
+
+@pytest.mark.parametrize("L,onsite,strips", [((150, 150), True, True), ((24, 25, 26), False, False)])
+def test_alternating_shapes_keep_their_plans(K, L, onsite, strips):
+    n = int(np.prod(L))
+    on = I.onsite_disorder(5, n, 2.0) if onsite else None
+    H = O.lattice_hamiltonian(L, onsite=on)
+    a, b = O.rescale(*O.gershgorin(H), eps=0.01)
+    M = 48
+    shapes = [(16, 4), (1, 4), (16, 3), (1, 3), (2, 4)]
+    with K.kpm_create_stencil(len(L), L, onsite=on) as h:
+        def call(S, R):
+            return K.kpm_moments(h, M, R, a, b, seed=3, S=S, per_vec=True)[1], K.kpm_testing_last_step_form(h)
+
+        first = [call(*s) for s in shapes]
+        assert {f for _, f in first} == ({"column strips", "fused step"} if strips else {"fused step"})
+        K.kpm_testing_fail_allocations(0)
+        try:
+            for _ in range(3):
+                for s, (pv, form) in zip(shapes, first):
+                    again, f = call(*s)
+                    assert f == form and np.array_equal(again, pv), s
+        finally:
+            K.kpm_testing_fail_allocations(-1)
+        # more shapes than are kept, and the first ones again
+        for S in range(3, 11):
+            assert np.abs(call(S, 4)[0] - first[0][0][:4 * S]).max() <= 1e-12
+        for s, (pv, _) in zip(shapes, first):
+            assert np.array_equal(call(*s)[0], pv), s
+    # each S against the same realisations alone
+    assert np.abs(first[0][0][:4] - first[1][0]).max() <= 1e-12
+    assert np.abs(first[0][0][:8] - first[4][0]).max() <= 1e-12
+
+
+@pytest.mark.parametrize("S", [2, 16])
+def test_large_lattice_beside_a_fixed_point_chain(K, S):
+    """90,000 sites: a chain in fixed point (unit 2^-52), column tasks on the FP64 pipe."""
+    L, M, R = (300, 300), 24, 2
+    on = I.onsite_disorder(6, 90000, 2.0)
+    H = O.lattice_hamiltonian(L, onsite=on)
+    a, b = O.rescale(*O.gershgorin(H), eps=0.01)
+    with K.kpm_create_stencil(2, L, onsite=on) as h:
+        for _ in range(2):
+            _, pv = K.kpm_moments(h, M, R, a, b, seed=4, S=S, per_vec=True)
+            _, one = K.kpm_moments(h, M, R, a, b, seed=4, per_vec=True)
+            assert np.abs(pv[:R] - one).max() <= 1e-12
+    for s in (0, S - 1):
+        per = O.moments_doubling(H, a, b, I.rademacher_block(4, H.n, R, s=s), M)[1]
+        assert np.abs(pv[s * R:(s + 1) * R] - per).max() <= 1e-10
