@@ -193,11 +193,14 @@ typedef struct {
  * complex one) with start blocks made by the library hold the vectors in 64-bit
  * fixed point when the scaled coefficients fit the format: the same absolute
  * resolution, off the slow FP64 pipe; KPM_FIXED=0, read when a call plans its
- * launches, keeps that pipe.  Returns KPM_EDIVERGE (after writing
- * the outputs) when host outputs show |mu_n^r| > 1 + 1e-6 or a non-finite
- * value, and KPM_EINVAL when R exceeds one block of vectors (more than 1024
- * chunks of 16 bytes (FP64) or 32 bytes (FP32) per row, after rounding the
- * chunk count up to a power of two; dense handles have no such limit). */
+ * launches, keeps that pipe.  An entry that leaves the format's range (the bounds
+ * miss the spectrum, and |v_n| has passed sqrt(N)) makes the moments of that
+ * product and of the later ones NaN, into host and device outputs alike.  Returns
+ * KPM_EDIVERGE (after writing the outputs) when host outputs show
+ * |mu_n^r| > 1 + 1e-6 or a non-finite value, and KPM_EINVAL when R exceeds one
+ * block of vectors (more than 1024 chunks of 16 bytes (FP64) or 32 bytes (FP32)
+ * per row, after rounding the chunk count up to a power of two; dense handles
+ * have no such limit). */
 kpm_status kpm_moments(kpm_handle h, const kpm_params* p, double* mu, double* mu_per_vec,
                        void* stream);
 

@@ -4,6 +4,7 @@
 // into a CUDA graph and replays it; every arithmetic step runs in the kernels
 // of kpm_step_*.cu and kpm_aux.cu.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stddef.h>
 #include <stdio.h>
@@ -265,6 +266,7 @@ StepArgs base_args(const kpm_handle_s* h, int slot, int Rp, int G) {
   a.sc = h->d_sc + slot;
   a.geom = h->geom;
   a.err = &h->d_prm->flags;
+  static_assert(offsetof(RunParams, bad_from) == offsetof(RunParams, flags) + sizeof(int));  // err[1]
   if (h->stencil) {
     a.hs = h->has_hop ? h->d_hs[slot] : nullptr;
     a.ds = h->has_onsite ? h->d_ds[slot] : nullptr;
@@ -1415,6 +1417,7 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
       a.w = w.v[(n + 1) & 1];
       a.partial = w.ring + (size_t)(n % RING) * grid * 2 * Rp;
       a.reverse = (n & 1) ^ 1;
+      a.step = n;
       e = launch_op(h, fp32, MODE_STEP, a, cfg, cs);
       if (e != cudaSuccess) break;
       if ((n + 1) % RING == 0)
@@ -1546,6 +1549,7 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
   prm.S = S;
   prm.M = M;
   prm.flags = 0;
+  prm.bad_from = INT_MAX;
   KPM_CUDA(cudaMemcpyAsync(h->d_prm, &prm, sizeof(prm), cudaMemcpyHostToDevice, st));
   // the operator scaled with this call's (a, b): kept from the previous call
   // on the same stream when that used the same (a, b)
@@ -1830,7 +1834,7 @@ kpm_status kpm_moments_extend(kpm_handle h, int M, double* mu, double* mu_per_ve
   prm.S = 1;
   prm.M = M;
   prm.flags = 0;
-  // (a fixed-point value out of range in an earlier call stays flagged)
+  // (a fixed-point value out of range in an earlier call stays flagged, with its product)
   KPM_CUDA(cudaMemcpyAsync(h->d_prm, &prm, w.proto.fixq > 0 ? offsetof(RunParams, flags) : sizeof(prm),
                            cudaMemcpyHostToDevice, st));
   // the same step launches as the uninterrupted chain: product n reads v_n
@@ -1852,6 +1856,7 @@ kpm_status kpm_moments_extend(kpm_handle h, int M, double* mu, double* mu_per_ve
     a.w = w.v[(n + 1) & 1];
     a.partial = w.ring + (size_t)(n % RING) * grid * 2 * Rp;
     a.reverse = (n & 1) ^ 1;
+    a.step = n;
     KPM_CUDA(launch_op(h, fp32, MODE_STEP, a, cfg, st));
     if ((n + 1) % RING == 0 || n == steps - 1) {
       const int first = std::max(old_steps, n / RING * RING);

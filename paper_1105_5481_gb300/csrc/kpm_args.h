@@ -36,7 +36,8 @@ struct RunParams {
   int R;                    // vectors per realisation
   int S;
   int M;
-  int flags;                // bit0: diverged
+  int flags;                // bit0: diverged; bits 2 and 3: see StepArgs::err
+  int bad_from;             // with bit 3: the first product whose result left its range
   int s0;                   // realisation index of s = 0 in the random-vector counters
 };
 
@@ -95,7 +96,8 @@ struct StepArgs {
                           // that many tiles ahead; < 0: none
   int tma_stall;          // testing aid: the producer issues no copy (the waits run out)
   int* err;               // bit 2 set by a bounded wait that ran out (may be NULL); bit 3 by a
-                          // fixed-point value out of range
+                          // fixed-point value out of range (err[1]: the least `step` of one)
+  int step;               // the product n (fixed point)
   int fixq;               // > 0: FP64 vectors held as 64-bit fixed point, 2^-fixq the unit
                           // (kpm_fixed.cuh)
 };

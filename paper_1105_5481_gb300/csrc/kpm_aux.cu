@@ -225,7 +225,9 @@ __global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* 
   const int step = blockIdx.x * FIN_STEPS + q;
   const int w = 2 * Rp, cols = S * R;
   const double inv_n = 1.0 / (double)n, lim = 1.0 + 1e-6;
-  const bool out_of_range = (prm->flags & 8) != 0;  // a fixed-point value left its range
+  // from the first fixed-point product whose result left its range on: v_{n+1}
+  // enters mu_{2n+1} and all that follow
+  const int bad_from = (prm->flags & 8) ? prm->bad_from : steps;
   double se = 0.0, so = 0.0;
   bool bad = false;
   if (step < steps) {
@@ -238,7 +240,8 @@ __global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* 
         me = 2.0 * base[(size_t)step * w + r] * inv_n - mu0;
         mo = 2.0 * base[(size_t)step * w + Rp + r] * inv_n - mu1;
       }
-      if (out_of_range) me = mo = NAN;
+      if (step > bad_from) me = NAN;
+      if (step >= bad_from) mo = NAN;
       double* pv = per_vec + (size_t)sr * M + 2 * step;
       pv[0] = me;
       pv[1] = mo;

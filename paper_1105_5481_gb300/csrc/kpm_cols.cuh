@@ -348,7 +348,7 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
 // the bonds of a site, where the FP64 pipe takes an FMA per bond at a 32nd of
 // that rate.  The dots' lane and warp sums are integer sums too.
 template <int DIMS, bool DS, int H, int G>
-__device__ __noinline__ void run_fixed(const ColsTask& k, int q, int C, int* err, unsigned char* smem) {
+__device__ __noinline__ void run_fixed(const ColsTask& k, int q, int C, unsigned char* smem) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int L = k.geom.L[DIMS - 1];
   const int U = k.geom.stride[DIMS - 1];
@@ -469,6 +469,7 @@ __device__ __noinline__ void run_fixed(const ColsTask& k, int q, int C, int* err
 
   const uint32_t bufb = (uint32_t)((size_t)bufn * 8);
   unsigned bad = 0;
+  int bad_from = nprod;  // the first product whose result left the range
   int bi = 0;
 #pragma unroll 1
   for (int m = 0; m < nprod; ++m) {
@@ -555,12 +556,17 @@ __device__ __noinline__ void run_fixed(const ColsTask& k, int q, int C, int* err
     if (C > 1) wait();
     else __syncthreads();
     if (m > 0 && m % kb == 0) bulk(m / kb - 1, kb);  // as in run_rows
+    if (bad) bad_from = min(bad_from, m);
     bi = bo;
   }
   if (C > 1) __syncthreads();
   const int bl = (nprod - 1) / kb;
   bulk(bl, nprod - bl * kb);
-  if (bad && err) atomicOr(err, 8);
+  if (bad && k.prm) {
+    RunParams* prm = const_cast<RunParams*>(k.prm);
+    atomicOr(&prm->flags, 8);
+    atomicMin(&prm->bad_from, bad_from);
+  }
 }
 
 // ------------------------------------------------------------------ FP32, slots
@@ -960,12 +966,11 @@ __global__ void __launch_bounds__(BT, 1)
       else if (hm <= 28) run_slots<DIMS, DS, 28, 4>(k, smem);
       else run_slots<DIMS, DS, 32, 4>(k, smem);
     } else if (k.fixq > 0) {
-      int* err = k.prm ? const_cast<int*>(&k.prm->flags) : k.flags;
-      if (hm <= 2) run_fixed<DIMS, DS, 2, 2>(k, q, C, err, smem);
-      else if (hm <= 4) run_fixed<DIMS, DS, 4, 2>(k, q, C, err, smem);
-      else if (hm <= 8) run_fixed<DIMS, DS, 8, 4>(k, q, C, err, smem);
-      else if (hm <= 12) run_fixed<DIMS, DS, 12, 4>(k, q, C, err, smem);
-      else run_fixed<DIMS, DS, 16, 4>(k, q, C, err, smem);
+      if (hm <= 2) run_fixed<DIMS, DS, 2, 2>(k, q, C, smem);
+      else if (hm <= 4) run_fixed<DIMS, DS, 4, 2>(k, q, C, smem);
+      else if (hm <= 8) run_fixed<DIMS, DS, 8, 4>(k, q, C, smem);
+      else if (hm <= 12) run_fixed<DIMS, DS, 12, 4>(k, q, C, smem);
+      else run_fixed<DIMS, DS, 16, 4>(k, q, C, smem);
     } else {
       if (hm <= 2) run_rows<DIMS, DS, 2, 2>(k, q, C, smem);
       else if (hm <= 4) run_rows<DIMS, DS, 4, 2>(k, q, C, smem);

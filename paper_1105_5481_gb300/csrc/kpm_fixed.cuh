@@ -39,7 +39,8 @@
 // 1.4, so real fields stay above (fixed_kind).  The dots are sums of exact
 // products likewise (<v_n|v_n> <= N bounds them), converted to FP64 once per
 // thread group.  A value past 2^61 (the spectrum is not enclosed: then a moment
-// has left [-1, 1] as well) sets bit 3 of the call's flags; the moments become NaN.
+// has left [-1, 1] as well) sets bit 3 of the call's flags; the moments that such a
+// product enters become NaN.
 #pragma once
 
 #include "kpm_step.cuh"
@@ -239,7 +240,10 @@ struct RowAcc<ChunkI64<CPLX>> {
     return __longlong_as_double((long long)(1023 + 64 - 2 * a.fixq) << 52);
   }
   static __device__ __forceinline__ void report(const StepArgs& a, unsigned bad) {
-    if (bad && a.err) atomicOr(a.err, 8);
+    if (bad && a.err) {
+      atomicOr(a.err, 8);
+      atomicMin(a.err + 1, a.step);
+    }
   }
 };
 
