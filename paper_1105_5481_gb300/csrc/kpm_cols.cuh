@@ -521,9 +521,11 @@ __device__ __noinline__ void run_fixed(const ColsTask& k, int q, int C, unsigned
             long long v = m == 0 ? (a11 << 3) + ((tt2 + (1ll << 24)) >> 25)
                                  : (a11 << 4) + ((tt2 + (1ll << 23)) >> 24);
             v -= w[j];
-            bad |= (unsigned)((int)(a11 >> 32) + (1 << 25)) > (1u << 26);
+            // (with a 64th to spare, as in kpm_fixed.cuh)
+            constexpr unsigned TOP = (1u << 25) + (1u << 19), X1 = (1u << 28) + (1u << 22);
+            bad |= (unsigned)(a11 >> 32) + TOP > 2 * TOP;
             const int v0 = (int)v, v1 = (int)((v - v0) >> 32);
-            bad |= (unsigned)(v1 + (1 << 28)) > (1u << 29);
+            bad |= (unsigned)v1 + X1 > 2 * X1;
             Y[j * U] = v;
             ah = mad64(u1, u1, ah);
             bh = mad64(v1, u1, bh);

@@ -38,9 +38,9 @@
 // rounding shows.  A real row has the fewest terms: at q = 51 it measured 0.6 to
 // 1.4, so real fields stay above (fixed_kind).  The dots are sums of exact
 // products likewise (<v_n|v_n> <= N bounds them), converted to FP64 once per
-// thread group.  A value past 2^61 (the spectrum is not enclosed: then a moment
-// has left [-1, 1] as well) sets bit 3 of the call's flags; the moments that such a
-// product enters become NaN.
+// thread group.  A value past 2^61 by a 64th (the spectrum is not enclosed: then a
+// moment has left [-1, 1] as well) sets bit 3 of the call's flags; the moments that
+// such a product enters become NaN.
 #pragma once
 
 #include "kpm_step.cuh"
@@ -216,7 +216,9 @@ struct RowAcc<ChunkI64<CPLX>> {
   static constexpr bool kIssueBound = true;
   static __device__ __forceinline__ void fold(type& r) { r.fold(); }
   // The sums rounded to the unit, less v_{n-1}.  `bad` is set when a value
-  // leaves +-2^61: |a11| bounds the sum before its shift can overflow.
+  // leaves +-2^61 by more than a 64th: |a11| bounds the sum before its shift can
+  // overflow.  (The start block of one site of N = 4^k lies on 2^61, and a spectrum
+  // outside the bounds by less than KPM_EDIVERGE allows for passes it by 2.5e-7.)
   static __device__ __forceinline__ CH done(const type& r, unsigned& bad) {
     CH y;
 #pragma unroll
@@ -231,8 +233,9 @@ struct RowAcc<ChunkI64<CPLX>> {
       const int lo = (int)v;
       y.x0[q] = lo;
       y.x1[q] = (int)((v - lo) >> 32);
-      bad |= (unsigned)(top + (1 << 26)) > (1u << 27);
-      bad |= (unsigned)(y.x1[q] + (1 << 29)) > (1u << 30);
+      constexpr unsigned TOP = (1u << 26) + (1u << 20), X1 = (1u << 29) + (1u << 23);
+      bad |= (unsigned)top + TOP > 2 * TOP;
+      bad |= (unsigned)y.x1[q] + X1 > 2 * X1;
     }
     return y;
   }

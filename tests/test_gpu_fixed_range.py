@@ -1,6 +1,7 @@
 """Fixed-point values that leave their range (bounds that miss the spectrum): the
 moments of the products before are kept, as on the FP64 pipe, the later ones are NaN,
-into device outputs too."""
+into device outputs too; and a spectrum outside the bounds by less than what
+KPM_EDIVERGE allows is none of it."""
 import numpy as np
 import pytest
 import torch
@@ -50,3 +51,19 @@ def test_moments_before_the_range_is_left(K, monkeypatch, L, S, R, form):
     m = int(ok.sum())
     assert 8 <= m < M and ok[:m].all() and not ok[m:].any()
     assert np.abs(fix[:m] / pipe[:m] - 1).max() <= 1e-9
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+def test_a_spectrum_just_outside_the_bounds(K, monkeypatch, cplx):
+    """Sites without bonds, the first 1e-10 outside: its entry grows past sqrt(N) =
+    2^6, the format's range, by 1e-7 while every moment stays within 1 + 1e-6."""
+    monkeypatch.setenv("KPM_COLRES", "0")
+    L, n, M = (64, 64), 4096, 64
+    x = np.linspace(-0.9, 0.9, n)
+    x[0] = 1.0 + 1e-10
+    with K.kpm_create_stencil(2, L, onsite=x, t=0.0, complex_=cplx) as h:
+        mu = K.kpm_ldos_moments(h, [0, 1, 4095], M, 1.0, 0.0, precision="fp64")
+    k = np.arange(M)
+    np.testing.assert_allclose(mu[0], np.cosh(k * np.arccosh(x[0])), rtol=0, atol=1e-12)
+    for j, i in ((1, 1), (2, 4095)):
+        np.testing.assert_allclose(mu[j], np.cos(k * np.arccos(x[i])), rtol=0, atol=1e-12)
