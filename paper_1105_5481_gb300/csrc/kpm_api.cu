@@ -1241,7 +1241,6 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps, int fixq,
       t.Rp = w.Rp;
       t.R = R;
       t.M = 2 * steps;
-      t.n1 = steps;
       if (C > 1) {
         t.part = (double*)(part * sizeof(double));  // made a pointer below
         part += (size_t)C * steps * 2 * (c1 - c0);

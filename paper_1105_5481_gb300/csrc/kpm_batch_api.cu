@@ -232,8 +232,6 @@ bool plan_cols(const kpm_batch_s* b, int C, ColsPlan* out) {
       t.n = bt.a.n;
       t.sc = bt.a.sc;
       t.ds = bt.a.ds;
-      t.v[0] = bt.v[0];
-      t.v[1] = bt.v[1];
       t.sums = bt.sums;
       t.seed = bt.seed;
       t.s = bt.realisation;
@@ -241,14 +239,12 @@ bool plan_cols(const kpm_batch_s* b, int C, ColsPlan* out) {
       t.R = bt.R;
       t.M = bt.M;
       cols_set_layout(t, s, b->fp32, c0, c1 - c0);
-      t.n0 = 0;
-      t.n1 = bt.M / 2;
       t.per_vec = bt.per_vec;
       t.mu = bt.mu;
       t.flags = b->d_queue + 1 + b->count + i;
       t.tiles_done = b->d_queue + 1 + i;
       t.ntiles = groups;
-      const double us = t.n1 * (s.us_fixed + t.ncol * s.us_col);
+      const double us = t.M / 2 * (s.us_fixed + t.ncol * s.us_col);
       total += us;
       p.us = std::max(p.us, us);
       p.smem = std::max(p.smem, cols_smem(s, b->fp32, t.ncol));
@@ -259,7 +255,7 @@ bool plan_cols(const kpm_batch_s* b, int C, ColsPlan* out) {
   for (Item& it : items) {
     if (C > 1) {
       it.t.part = (double*)(p.part * sizeof(double));  // offset, made a pointer when the scratch exists
-      p.part += (size_t)C * it.t.n1 * 2 * it.t.ncol;
+      p.part += (size_t)C * (it.t.M / 2) * 2 * it.t.ncol;
     }
     p.tasks.push_back(it.t);
   }
@@ -353,7 +349,7 @@ bool cols_faster(kpm_batch_s* b, int C) {
     const double sites = t.ncol * (t.tpc / 32) * t.height / 16.0;  // a scheduler's, in fours
     const double us = d3 ? 0.26 + 0.029 * t.height + 0.084 * sites + sweeps * (0.44 + 0.018 * rows)
                          : 0.22 + 0.017 * t.height + 0.071 * sites + sweeps * (0.49 + 0.011 * rows);
-    strips.push_back(us * t.n1);
+    strips.push_back(us * (t.M / 2));
   }
   return 1.15 * (20.0 + makespan(strips, p.clusters)) <= t_global;
 }

@@ -169,8 +169,7 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
     cbm = hb ? hu : T(0);
   }
 
-  // start vectors; the first product runs with halved coefficients
-  const bool first = k.n0 == 0;
+  // start vectors
   T x[H], w[H];
   {
     const unsigned long long seed = k.prm ? k.prm->seed : k.seed;
@@ -181,13 +180,8 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
       x[j] = w[j] = T(0);
       if (j < H - G ? act : j < h) {
         const int64_t i = (int64_t)(r0 + y0 + j) * U + u;
-        if (first && !k.start) {
-          T im;
-          random_value<T, false>(k.n, k.R, seed, s, i, col, x[j], im);
-        } else {
-          x[j] = reinterpret_cast<const T*>(k.v[k.n0 & 1])[i * k.Rp + col];
-          if (!first) w[j] = reinterpret_cast<const T*>(k.v[(k.n0 & 1) ^ 1])[i * k.Rp + col];
-        }
+        T im;
+        random_value<T, false>(k.n, k.R, seed, s, i, col, x[j], im);
         buf[base + j * U] = x[j];
         if (DS && cc == 0) dsm[base + j * U] = src[i];
       }
@@ -205,8 +199,9 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
       cb[d] *= f;
     }
   };
-  T df = first ? T(0.5) : T(1);  // scale of the diagonal in shared memory
-  if (first) scale(T(0.5));
+  // the first product runs with halved coefficients
+  T df = T(0.5);  // scale of the diagonal in shared memory
+  scale(T(0.5));
   auto sync = [&]() {
     if (C > 1) {
       arrive();
@@ -217,7 +212,7 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
   };
   sync();
 
-  const int nprod = k.n1 - k.n0;
+  const int nprod = k.M / 2;
   const int wpc = tpc >> 5;
   // the sums of `cnt` products of batch b
   auto bulk = [&](int b, int cnt) {
@@ -236,8 +231,8 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
         a += __shfl_xor_sync(0xffffffffu, a, 1);
         a += __shfl_xor_sync(0xffffffffu, a, 2);
         if (on && sub == 0) {
-          const int step = b * kb + pi;  // product n0 + step
-          if (C == 1) k.sums[(size_t)(k.n0 + step) * 2 * k.Rp + (size_t)dot * k.Rp + k.col0 + c] = a;
+          const int step = b * kb + pi;
+          if (C == 1) k.sums[(size_t)step * 2 * k.Rp + (size_t)dot * k.Rp + k.col0 + c] = a;
           else k.part[((size_t)q * nprod + step) * 2 * ncol + r] = a;
         }
       }
@@ -316,7 +311,7 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
       // written kb products later
       if (m > 0 && m % kb == 0) bulk(m / kb - 1, kb);
     }
-    if (m == 0 && first) {
+    if (m == 0) {
       scale(T(2));
       df = T(1);
     }
@@ -326,17 +321,6 @@ __device__ __noinline__ void run_rows(const ColsTask& k, int q, int C, unsigned 
     if (C > 1) __syncthreads();  // the ring entries of the last product
     const int bl = (nprod - 1) / kb;
     bulk(bl, nprod - bl * kb);
-  }
-  if (k.keep && act) {
-    T* va = reinterpret_cast<T*>(k.v[k.n1 & 1]);
-    T* vb = reinterpret_cast<T*>(k.v[(k.n1 & 1) ^ 1]);
-#pragma unroll
-    for (int j = 0; j < H; ++j)
-      if (j < H - G || j < h) {
-        const int64_t i = (int64_t)(r0 + y0 + j) * U + u;
-        va[i * k.Rp + col] = x[j];
-        vb[i * k.Rp + col] = w[j];
-      }
   }
 }
 
@@ -434,7 +418,7 @@ __device__ __noinline__ void run_fixed(const ColsTask& k, int q, int C, unsigned
   };
   sync();
 
-  const int nprod = k.n1;
+  const int nprod = k.M / 2;
   const int wpc = tpc >> 5;
   auto bulk = [&](int b, int cnt) {
     const int items = cnt * 2 * ncol;
@@ -736,8 +720,7 @@ __device__ __noinline__ void run_slots(const ColsTask& k, unsigned char* smem) {
     cbm = hb ? hu : 0.0f;
   }
 
-  // start vectors; the first product runs with halved coefficients
-  const bool first = k.n0 == 0;
+  // start vectors
   float x[H], dd[DS ? H : 1];
   {
     const unsigned long long seed = k.prm ? k.prm->seed : k.seed;
@@ -750,16 +733,10 @@ __device__ __noinline__ void run_slots(const ColsTask& k, unsigned char* smem) {
       if (j < H - G ? act : j < h) {
         const int64_t i = (int64_t)(y0 + j) * Ur + (x0 + yy * L0);
         if (DS) dd[j] = src[i];
-        float wj = 0.0f;
-        if (first && !k.start) {
-          float im;
-          random_value<float, false>(k.n, k.R, seed, s, i, col, x[j], im);
-        } else {
-          x[j] = reinterpret_cast<const float*>(k.v[k.n0 & 1])[i * k.Rp + col];
-          if (!first) wj = reinterpret_cast<const float*>(k.v[(k.n0 & 1) ^ 1])[i * k.Rp + col];
-        }
+        float im;
+        random_value<float, false>(k.n, k.R, seed, s, i, col, x[j], im);
         buf[j * SLOT + t] = x[j];
-        buf[2 * bufn + j * SLOT + t] = wj;
+        buf[2 * bufn + j * SLOT + t] = 0.0f;
       }
     }
   }
@@ -797,17 +774,17 @@ __device__ __noinline__ void run_slots(const ColsTask& k, unsigned char* smem) {
       for (int j = 0; j < H; ++j) dd[j] *= f;
     }
   };
-  if (first) scale(0.5f);
+  scale(0.5f);  // the first product runs with halved coefficients
   __syncthreads();
 
-  const int nprod = k.n1 - k.n0;
+  const int nprod = k.M / 2;
   const int gl = 1 << (o.lg - 3);  // chains per group
   auto bulk = [&](int b, int cnt) {
     const int items = cnt * 2 * ncol;
     const float2* rb = ring + (b & 1) * kb * ncol * rentry;
     for (int it = t; it < items; it += BT) {
       const int pi = it / (2 * ncol), r = it - pi * 2 * ncol, c = r >> 1, dot = r & 1;
-      k.sums[(size_t)(k.n0 + b * kb + pi) * 2 * k.Rp + (size_t)dot * k.Rp + k.col0 + c] =
+      k.sums[(size_t)(b * kb + pi) * 2 * k.Rp + (size_t)dot * k.Rp + k.col0 + c] =
           slot_total(rb + (pi * ncol + c) * rentry, o.NR, dot);
     }
   };
@@ -902,24 +879,12 @@ __device__ __noinline__ void run_slots(const ColsTask& k, unsigned char* smem) {
       if (m > kb && ((m - 1) & (kb - 1)) == 0) bulk(((m - 1) >> kl) - 1, kb);
     }
     __syncthreads();
-    if (m == 0 && first) scale(2.0f);
+    if (m == 0) scale(2.0f);
     bi = bo;
   }
   // the batch not summed in the loop (its last phase is that of product nprod)
   const int bl = (nprod - 1) / kb;
   bulk(bl, nprod - bl * kb);
-  if (k.keep && act) {
-    float* va = reinterpret_cast<float*>(k.v[k.n1 & 1]);
-    float* vb = reinterpret_cast<float*>(k.v[(k.n1 & 1) ^ 1]);
-    const float* W = buf + (nprod - 1) % 3 * bufn + t;
-#pragma unroll
-    for (int j = 0; j < H; ++j)
-      if (j < H - G || j < h) {
-        const int64_t i = (int64_t)(y0 + j) * Ur + (x0 + yy * L0);
-        va[i * k.Rp + col] = x[j];
-        vb[i * k.Rp + col] = W[j * SLOT];
-      }
-  }
 }
 
 template <typename T, int DIMS, bool DS>
@@ -980,7 +945,7 @@ __global__ void __launch_bounds__(BT, 1)
       else if (hm <= 12) run_rows<DIMS, DS, 12, 4>(k, q, C, smem);
       else run_rows<DIMS, DS, 16, 4>(k, q, C, smem);
     }
-    const int nprod = k.n1 - k.n0, ncol = k.ncol;
+    const int nprod = k.M / 2, ncol = k.ncol;
     if (C > 1) {
       // the CTAs' partials, added in rank order
       arrive();
@@ -990,18 +955,17 @@ __global__ void __launch_bounds__(BT, 1)
         const int step = e / (2 * ncol), r = e - step * 2 * ncol;
         double s = 0.0;
         for (int p = 0; p < C; ++p) s += k.part[(size_t)p * total + e];
-        k.sums[(size_t)(k.n0 + step) * 2 * k.Rp + (size_t)(r & 1) * k.Rp + k.col0 + (r >> 1)] = s;
+        k.sums[(size_t)step * 2 * k.Rp + (size_t)(r & 1) * k.Rp + k.col0 + (r >> 1)] = s;
       }
       arrive();
       wait();
     }
     __syncthreads();  // the sums of this task (C == 1: written by this CTA)
-    const int nsteps = k.M / 2;
-    if (k.per_vec && k.n1 == nsteps && q == 0) {
+    if (k.per_vec && q == 0) {
       const int M = k.M, R = k.R, Rp = k.Rp;
       const double inv_n = 1.0 / (double)k.n;
-      for (int e = t; e < ncol * nsteps; e += BT) {
-        const int r = k.col0 + e / nsteps, step = e % nsteps;
+      for (int e = t; e < ncol * nprod; e += BT) {
+        const int r = k.col0 + e / nprod, step = e % nprod;
         const double mu0 = k.sums[r] * inv_n, mu1 = k.sums[Rp + r] * inv_n;
         double me = mu0, mo = mu1;
         if (step > 0) {

@@ -39,9 +39,8 @@ struct ColsTask {
   int64_t n;
   const ScalarBlock* sc;
   const void* ds;             // scaled diagonal [N], or NULL (uniform)
-  void* v[2];                 // N x Rp vector blocks (read or written as start and keep say)
   double* sums;               // [steps][2][Rp] per-step sums over rows of this realisation
-  double* part;               // C > 1: [C][n1 - n0][2 ncol] scratch
+  double* part;               // C > 1: [C][M / 2][2 ncol] scratch
   const RunParams* prm;       // not NULL: seed and first realisation are read from here
   unsigned long long seed;
   long long s;                // realisation (added to prm->s0 when prm is given)
@@ -50,10 +49,7 @@ struct ColsTask {
   int strips, height, tpc, rows, pitch, spi, lines;  // ColsShape
   int batch;                  // products per batch of the dot sums
   int fixq;                   // FP64, > 0: 64-bit fixed point of unit 2^-fixq (kpm_fixed.cuh;
-                              // ds in its format, whole solves from drawn vectors)
-  int n0, n1;                 // products n0 .. n1-1 (product n reads v_n, writes v_{n+1})
-  int start;                  // n0 == 0: 0 draws v_0, 1 loads it from v[0]
-  int keep;                   // store v_{n1-1} and v_{n1} at the end
+                              // ds in its format)
   // finalisation in the kernel (batches): the instance's per-vector moments
   // and mean, written by the last of its `ntiles` tasks; per_vec NULL: none
   double* per_vec;
