@@ -238,13 +238,19 @@ void free_cols(kpm_handle_s::Work& w) {
   w.cs_now = -1;
 }
 
+void free_chain(kpm_handle_s::Chain& c) {
+  if (c.exec) cudaGraphExecDestroy(c.exec);
+  dfree(c.ring);
+  c = {};
+}
+
 void free_work(kpm_handle_s* h) {
   auto& w = h->work;
-  if (w.exec) cudaGraphExecDestroy(w.exec);
+  free_chain(w);
+  free_chain(w.other);
   free_dense_tc(w);
   dfree(w.v[0]);
   dfree(w.v[1]);
-  dfree(w.ring);
   dfree(w.sums);
   dfree(w.per_vec);  // w.mu points into per_vec
   dfree(w.v0stage);
@@ -1360,17 +1366,40 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
   kpm_status s_ = ensure_scaled(h, slot, fp32);
   if (s_ != KPM_OK) return s_;
 
-  // the step chain in fixed point, decided when it is planned and again when
-  // a call's kind or (a, b) would decide otherwise
   const bool fix_kind = fixed_kind(h, fp32, p);
-  const int unit_now = fix_kind && h->ranged ? fixed_unit(h, p->a, p->b) : 0;
   const size_t sums_bytes = (size_t)S * steps * 2 * Rp * sizeof(double);
   const size_t out_bytes = ((size_t)S * R * M + M) * sizeof(double);
   const bool rebuild = w.Rp != Rp || w.prec != p->precision || w.M != M ||
                        w.user_v0 != user_v0 || !w.ready || w.sums_bytes < sums_bytes ||
-                       (w.cr.C > 0 && w.cr_R != R) ||
-                       (!h->dense && w.cr.C == 0 &&
-                        (w.proto.fixq > 0) != (h->ranged ? unit_now > 0 && !w.fix_off : fix_kind && w.proto.fixq > 0));
+                       (w.cr.C > 0 && w.cr_R != R);
+  // the unit of the step chain in fixed point, 0 for the FP64 pipe (also without
+  // memory for the operator's second copy)
+  auto chain_unit = [&](int* q) -> kpm_status {
+    *q = 0;
+    if (!fix_kind || w.fix_off || w.cr.C > 0) return KPM_OK;
+    kpm_status sa = ensure_range(h);
+    if (sa == KPM_OK && (*q = fixed_unit(h, p->a, p->b)) > 0) sa = ensure_fixed(h);
+    if (sa != KPM_OK) *q = 0;
+    if (sa != KPM_ENOMEM) return sa;
+    w.fix_off = true;
+    return KPM_OK;
+  };
+  // the launches of unit q (0: FP64 pipe or FP32) as the chain in use
+  auto plan_chain = [&](StepArgs a, int block, int grid, int q) -> kpm_status {
+    if (q > 0) {
+      a.fixq = q;
+      if (!h->stencil) a.vals = h->d_hs_fix;
+      else if (h->has_hop) a.hs = h->d_hs_fix;
+      if (h->has_onsite) a.ds = h->d_ds_fix;
+      plan_grid(h, fp32, a, &block, &grid);
+    }
+    w.proto = a;
+    w.nCTA = grid;
+    w.block = block;
+    kpm_status sa = dalloc(&w.ring, (size_t)RING * grid * 2 * Rp);
+    w.planned = sa == KPM_OK;
+    return sa;
+  };
   // The kernel sequence of one realisation.  The first call of a shape
   // launches it directly on the caller's stream (the solve is GPU-bound, so
   // the launches hide behind it); a second call of the same shape captures it
@@ -1432,10 +1461,8 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
   };
   if (rebuild) {
     KPM_CUDA(cudaDeviceSynchronize());
-    if (w.exec) {
-      cudaGraphExecDestroy(w.exec);
-      w.exec = nullptr;
-    }
+    free_chain(w);
+    free_chain(w.other);
     // buffers are about to be replaced: until the plan below is complete no
     // later call may take the old one (an allocation failing half way leaves
     // the handle to rebuild on its next call)
@@ -1469,7 +1496,6 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     StepArgs proto = base_args(h, slot, Rp, G);
     int block, grid;
     plan_grid(h, fp32, proto, &block, &grid);
-    w.proto = proto;
     // small stencil and padded-ELL operators: the column-resident solve
     // replaces the chain of step launches (unless a TMA-fed step was planned)
     w.cr = ColresPlan{};
@@ -1487,38 +1513,37 @@ kpm_status moments_impl(kpm_handle h, const kpm_params* p, double* mu, double* m
     else free_dense_tc(w);
     w.Rp = Rp;
     free_cols(w);
-    if (fix_kind && w.cr.C == 0) {
-      // (without memory for the operator's second copy: the FP64 pipe)
-      kpm_status sa = ensure_range(h);
-      const int q = sa == KPM_OK ? fixed_unit(h, p->a, p->b) : 0;
-      if (q > 0) sa = ensure_fixed(h);
-      if (sa == KPM_ENOMEM) w.fix_off = true;
-      else if (sa != KPM_OK) return sa;
-      else if (q > 0) {
-        w.proto.fixq = q;
-        if (!h->stencil) w.proto.vals = h->d_hs_fix;
-        else if (h->has_hop) w.proto.hs = h->d_hs_fix;
-        if (h->has_onsite) w.proto.ds = h->d_ds_fix;
-        plan_grid(h, fp32, w.proto, &block, &grid);
-      }
-    }
-    dfree(w.ring);
-    w.ring = nullptr;
-    {
-      kpm_status sa = dalloc(&w.ring, (size_t)RING * grid * 2 * Rp);
-      if (sa != KPM_OK) return sa;
-    }
+    int q = 0;
+    kpm_status sa = chain_unit(&q);
+    if (sa == KPM_OK) sa = plan_chain(proto, block, grid, q);
+    if (sa != KPM_OK) return sa;
     w.Rp = Rp;
     w.prec = p->precision;
     w.M = M;
     w.user_v0 = user_v0;
-    w.nCTA = grid;
-    w.block = block;
     if (!w.ev[0]) KPM_CUDA(cudaEventCreate(&w.ev[0]));
     if (!w.ev[1]) KPM_CUDA(cudaEventCreate(&w.ev[1]));
     w.timed = false;
     w.ready = true;
-    w.direct_done = false;
+  } else if (!h->dense && w.cr.C == 0) {
+    // the other arithmetic where this call's start block or (a, b) take it; its
+    // launches are planned once and stand beside these
+    int q = 0;
+    kpm_status sa = chain_unit(&q);
+    if (sa != KPM_OK) return sa;
+    if ((w.proto.fixq > 0) != (q > 0)) {
+      std::swap<kpm_handle_s::Chain>(w, w.other);
+      if (!w.planned) {
+        StepArgs proto = base_args(h, slot, Rp, G);
+        int block, grid;
+        plan_grid(h, fp32, proto, &block, &grid);
+        sa = plan_chain(proto, block, grid, q);
+        if (sa != KPM_OK) {
+          std::swap<kpm_handle_s::Chain>(w, w.other);
+          return sa;
+        }
+      }
+    }
   }
   s_ = cols_solve(h, p, R, S, steps, fix_kind, st);
   if (s_ != KPM_OK) return s_;

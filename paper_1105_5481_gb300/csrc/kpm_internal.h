@@ -295,13 +295,25 @@ struct kpm_handle_s {
   void* scaled_st[2] = {nullptr, nullptr};
   kpm::RunParams* d_prm = nullptr;
   // moments workspace
-  struct Work {
-    int Rp = 0, prec = -1, M = 0, nCTA = 0, block = 0;
+  // the step chain's launches in one arithmetic
+  struct Chain {
+    kpm::StepArgs proto{};  // launch arguments common to all steps
+    int nCTA = 0, block = 0;
+    double* ring = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    uint64_t kernels_per_replay = 0;
+    bool direct_done = false;  // one call of this shape ran without a graph
+    bool planned = false;
+  };
+  struct Work : Chain {
+    // the chain not in use (FP64 pipe and fixed point; calls that alternate between
+    // start blocks or (a, b) of either kind replace neither)
+    Chain other;
+    int Rp = 0, prec = -1, M = 0;
     bool fix_off = false;  // no memory for this plan's fixed-point operator
     bool user_v0 = false;
     void* v[2] = {nullptr, nullptr};
     size_t vbytes = 0;
-    double* ring = nullptr;
     double* sums = nullptr;
     size_t sums_bytes = 0;
     double* per_vec = nullptr;
@@ -311,11 +323,7 @@ struct kpm_handle_s {
     size_t v0stage_bytes = 0;
     void* sb_dev = nullptr;   // parameters of a device-built start block
     size_t sb_bytes = 0;
-    cudaGraphExec_t exec = nullptr;
-    uint64_t kernels_per_replay = 0;
-    bool ready = false;        // buffers and launch plan match the current shape
-    bool direct_done = false;  // one call of this shape ran without a graph
-    kpm::StepArgs proto{};                    // launch arguments common to all steps
+    bool ready = false;  // buffers and launch plan match the current shape
     // the dense product on the tensor cores (real FP64 dense handles)
     kpm::DenseTC* dtc = nullptr;
     // resumable state of the last kpm_moments call (S == 1): v_{n-1}, v_n in

@@ -1,6 +1,7 @@
 """Plans that stand beside each other: calls that alternate the realisations S, or
-the vectors R within one padded width, replace none of them (nothing is allocated
-when a shape comes again) and keep their bits; the column tasks of an operator too
+the vectors R within one padded width, or start blocks of the caller's and of the
+library's making, replace none of them (nothing is allocated when a shape comes again)
+and keep their bits; the column tasks of an operator too
 large for their fixed-point unit run beside a step chain in fixed point."""
 import numpy as np
 import pytest
@@ -48,6 +49,35 @@ def test_alternating_shapes_keep_their_plans(K, L, onsite, strips):
     # each S against the same realisations alone
     assert np.abs(first[0][0][:4] - first[1][0]).max() <= 1e-12
     assert np.abs(first[0][0][:8] - first[4][0]).max() <= 1e-12
+
+
+@pytest.mark.parametrize("user_first", [False, True])
+def test_alternating_start_blocks_keep_their_plans(K, user_first):
+    """A user's start block on the FP64 pipe, one of sites in fixed point."""
+    L, M = (150, 150), 48
+    on = I.onsite_disorder(5, 22500, 2.0)
+    H = O.lattice_hamiltonian(L, onsite=on)
+    a, b = O.rescale(*O.gershgorin(H), eps=0.01)
+    v0 = I.random_block(7, H.n, 4, False)
+    sites = [0, 77, 11111, 22499]
+    with K.kpm_create_stencil(2, L, onsite=on) as h:
+        def call(user):
+            if user:
+                return K.kpm_moments(h, M, 4, a, b, user_v0=v0, per_vec=True)[1]
+            return K.kpm_ldos_moments(h, sites, M, a, b, precision="fp64")
+
+        first = {user: call(user) for user in (user_first, not user_first)}
+        K.kpm_testing_fail_allocations(0)
+        try:
+            for _ in range(3):
+                for user in (True, False):
+                    assert np.array_equal(call(user), first[user])
+        finally:
+            K.kpm_testing_fail_allocations(-1)
+    assert np.abs(first[True] - O.moments_doubling(H, a, b, v0, M)[1]).max() <= 1e-10
+    unit = np.zeros((H.n, 4))
+    unit[sites, np.arange(4)] = np.sqrt(H.n)
+    assert np.abs(first[False] - O.moments_doubling(H, a, b, unit, M)[1]).max() <= 1e-10
 
 
 @pytest.mark.parametrize("S", [2, 16])
