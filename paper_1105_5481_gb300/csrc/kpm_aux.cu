@@ -1066,6 +1066,18 @@ __device__ __forceinline__ double damping(int n, int M, int kernel, double lambd
 // clock; a 256-thread block of cos/sin on one SM took about 12 us for M = 256).
 constexpr int FP64_SPREAD = 32;
 
+// cos(pi j / (2K)), 0 <= j < 4K, to its own relative accuracy: the integer j is
+// reduced to the first octant, because the table's sines divide the density of states
+// and those next to the edges of the spectrum are of order 1 / K (cospi of j / (2K),
+// rounded near 1/2 or 3/2, is off by up to 3 K 2^-53 of them: 1.2e-12 at K = 8000).
+__device__ __forceinline__ double cos_node(int64_t j, int64_t K) {
+  int64_t r = j <= 2 * K ? j : 4 * K - j;
+  const bool neg = r > K;
+  if (neg) r = 2 * K - r;
+  const double v = 2 * r > K ? sinpi((double)(K - r) / (2.0 * (double)K)) : cospi((double)r / (2.0 * (double)K));
+  return neg ? -v : v;
+}
+
 // The damped coefficients coef[n] = c_n g_n mu_n (mu NULL: 1) and the cosine
 // table[j] = cos(pi j / (2K)), j = 0 .. 4K-1 (exact argument reduction for the
 // sums): independent of each other, one launch.
@@ -1080,7 +1092,7 @@ __global__ void dos_prep_kernel(const double* __restrict__ mu, int M, int kernel
       const double cotq = cos(q) / sin(q);
       coef[n] = (n == 0 ? 1.0 : 2.0) * damping(n, M, kernel, lambda, cotq) * (mu ? mu[n] : 1.0);
     } else {
-      table[e - M] = cospi((double)(e - M) / (2.0 * (double)K));
+      table[e - M] = cos_node(e - M, K);
     }
   }
 }
@@ -1142,8 +1154,7 @@ __global__ void green_kernel(const double* __restrict__ coef, int M, double a, d
     sn += __shfl_xor_sync(0xffffffffu, sn, o);
   }
   if (lane == 0) {
-    double sx, cx;
-    sincospi(((double)warp + 0.5) / (double)K, &sx, &cx);
+    const double cx = table[step], sx = table[(step + k3) % n4];
     if (E) E[warp] = a * cx + b;
     g_re[warp] = -sn / (a * sx);
     g_im[warp] = -c / (a * sx);
