@@ -18,9 +18,10 @@
 // The sums fit: sum |h| <= 15 over a row, which the host checks, bounds h1 x1 and
 // h1 x0 by 2^63 for any number of entries.  h0 does not shrink with h (|h0| <= 2^27,
 // |x0| <= 2^31), so h0 x0 holds 31 products and h0 x1 127: stencil rows have at most
-// 13 of each per component, padded rows 17, and CSR rows of any length carry the
-// upper parts of both classes to the next one every 8 entries (Row::fold; at most 17
-// products lie between).
+// 13 of each per component, padded rows 17, and the entries of a CSR row beyond 30
+// (15 in complex fields) are followed, four by four, by carries of the upper parts to
+// the next class (Row::fold).  (Carries within every row, each 8 or 16 entries, cost
+// rows of up to 19 entries 2 to 5 %.)
 //
 // Measured (3D L = 64 spin lattice, 64 complex vectors): 374 us per step against
 // 939 on the FP64 pipe.  Bound by issue at 16 warps per SM (math-pipe throttle
@@ -214,6 +215,8 @@ struct RowAcc<ChunkI64<CPLX>> {
   using CH = ChunkI64<CPLX>;
   using type = typename CH::Row;
   static constexpr bool kIssueBound = true;
+  // (31 products, the diagonal's among them)
+  static constexpr int kFold = CPLX ? 15 : 30;
   static __device__ __forceinline__ void fold(type& r) { r.fold(); }
   // The sums rounded to the unit, less v_{n-1}.  `bad` is set when a value
   // leaves +-2^61 by more than a 64th: |a11| bounds the sum before its shift can

@@ -322,14 +322,14 @@ __device__ __forceinline__ ScalPair<double> ldg_pair(const double* p, size_t i) 
 }
 
 // The accumulator of one row's chunk (the chunk itself unless it says
-// otherwise), the chunk it ends in, and the factor of its dots.  fold is called
-// at least once per 8 entries of a CSR row.  kIssueBound: instructions, not
-// accesses in flight, limit the step.
+// otherwise), the chunk it ends in, and the factor of its dots.  kIssueBound:
+// instructions, not accesses in flight, limit the step.  kFold > 0: at most that many
+// entries of a CSR row are added up without a call of fold(acc).
 template <class CH, class = void>
 struct RowAcc {
   using type = CH;
   static constexpr bool kIssueBound = false;
-  static __device__ __forceinline__ void fold(CH&) {}
+  static constexpr int kFold = 0;
   static __device__ __forceinline__ const CH& done(const CH& acc, unsigned&) { return acc; }
   static __device__ __forceinline__ double dot_scale(const StepArgs&) { return 1.0; }
   static __device__ __forceinline__ void report(const StepArgs&, unsigned) {}
@@ -557,6 +557,7 @@ struct CsrOp {
   static constexpr bool kCanAhead = CH::NC && !std::is_same<T, double>::value;
   static constexpr int kMinBlocks = AHEAD || !std::is_same<Row, CH>::value ? 2 : KPM_SPARSE_MIN_BLOCKS;
   static constexpr bool kPairReduce = false;
+  static constexpr int kFold = RowAcc<CH>::kFold;
   struct LineCtx {};
   __device__ __forceinline__ void hop(const T* V, int64_t k, T& hr, T& hi) const {
     if constexpr (CPLX) {
@@ -589,7 +590,7 @@ struct CsrOp {
           }
       };
       fetch(0);
-      for (int k = 0; k < len; k += B) {
+      auto batch = [&](int k) {
         CH xj[B];
 #pragma unroll
         for (int u = 0; u < B; ++u)
@@ -604,11 +605,19 @@ struct CsrOp {
 #pragma unroll
         for (int u = 0; u < B; ++u)
           if (k + u < len) acc.cmac(cr[u], ci[u], xj[u]);
-        if (k & 4) RowAcc<CH>::fold(acc);
+      };
+      int k = 0;
+      if constexpr (kFold > 0) {
+#pragma unroll 1
+        for (; len - k > kFold; k += B) {
+          batch(k);
+          RowAcc<CH>::fold(acc);
+        }
       }
+      for (; k < len; k += B) batch(k);
     } else {
       int64_t k = k0;
-      for (; k + 4 <= k1; k += 4) {
+      auto batch = [&]() {
         int j[4];
         T hr[4], hi[4];
 #pragma unroll
@@ -621,8 +630,15 @@ struct CsrOp {
         for (int u = 0; u < 4; ++u) xj[u].ld_x(Xc + (size_t)j[u] * rowS);
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc.cmac(hr[u], hi[u], xj[u]);
-        if ((k - k0) & 4) RowAcc<CH>::fold(acc);
+      };
+      if constexpr (kFold > 0) {
+#pragma unroll 1
+        for (; k1 - k > kFold; k += 4) {
+          batch();
+          RowAcc<CH>::fold(acc);
+        }
       }
+      for (; k + 4 <= k1; k += 4) batch();
       for (; k < k1; ++k) {
         const int j = __ldg(a.col + k);
         T hr, hi;
