@@ -26,7 +26,11 @@ namespace kpm {
 
 // Largest operators whose FP64 vectors go into 64-bit fixed point: the unit is
 // 2^-52 or finer for real fields, 2^-51 for complex ones (whose rows have four
-// times the terms, each with its rounding, on the FP64 pipe).
+// times the terms, each with its rounding, on the FP64 pipe).  Root mean square error
+// of the moments against 64-bit significands, over the FP64 pipe's (M = 64, 8
+// vectors): complex at 2^-51 0.93 (3D, 524,800 sites), 1.02 (3D, 388,944), 0.95 (3D,
+// 1,040,502), 1.01 (2D, 1,043,460), at 2^-52 0.99 (3D, 262,144); real at 2^-52 0.97
+// (2D, 261,632), 0.91 (3D, 262,080), and at 2^-51 0.6 to 1.4.
 constexpr int64_t FIXED_MAX_N_REAL = 1 << 18, FIXED_MAX_N_CPLX = 1 << 20;
 
 // vector columns per chunk (FP32: 32-byte chunks; FP64: 16-byte chunks)
@@ -702,8 +706,11 @@ bool columns_in_range(const int32_t* col, int64_t nnz, int64_t n) {
 
 using namespace kpm;
 
-// Smallest dimension whose Lanczos vectors are reorthogonalised only where
-// needed.
+// Smallest dimension whose Lanczos vectors are reorthogonalised only where needed:
+// there it is faster for 30 steps and more, and 10 steps are not slower.  kpm_bounds of
+// 3D lattices, 10 / 30 / 100 steps: 64,000 rows with the pass in every step 0.54 / 1.66
+// / 8.45 ms real, 0.68 / 2.31 / 13.5 complex; 85,184 rows where needed 0.59 / 1.60 /
+// 5.06 and 0.65 / 1.71 / 6.17.
 constexpr int64_t LANCZOS_PARTIAL_MIN_N = 1 << 16;
 
 extern "C" {
@@ -1183,6 +1190,9 @@ kpm_status ensure_fixed(kpm_handle_s* h) {
 // 256: 17.7 ms one after the other, 4.9 ms in one launch on the FP64 pipe, 2.0
 // in fixed point).  FP32 vectors keep the
 // solves in turn: their compensated dots depend on the form's sum order.
+// Against the step chain in fixed point (M = 64; 2D 16 to 510 a side, 3D 8 to 60; R of
+// 1, 4, 16; S of 2 to 64): taken in 154 of 233 shapes, where the tasks are 1.3 to 82
+// times as fast (median 5.4).
 bool cols_solve_kind(const kpm_handle_s* h, bool fp32) {
   return !fp32 && h->stencil && !h->cplx && !h->has_hop && (h->geom.dims == 2 || h->geom.dims == 3);
 }
@@ -1253,14 +1263,31 @@ kpm_status plan_cols_solve(kpm_handle_s* h, int R, int S, int steps, int fixq,
       }
       tasks.push_back(t);
     }
-  kpm_status sa = dalloc((char**)&cs.tasks, tasks.size() * sizeof(ColsTask));
-  if (sa == KPM_OK) sa = dalloc(&cs.queue, (size_t)1);
-  if (sa == KPM_OK && part) sa = dalloc(&cs.part, part);
-  if (sa != KPM_OK) {
-    free_cols(cs);
-    // the solves in turn need none of it (a later call tries again)
-    return sa == KPM_ENOMEM ? KPM_OK : sa;
-  }
+  // the kept launches of other (S, R) give way where this one's scratch is large, or
+  // where there is no memory beside them
+  auto drop_others = [&]() -> kpm_status {
+    bool any = false;
+    for (auto& o : w.cs) any |= &o != &cs && o.tasks;
+    if (!any) return KPM_ENOMEM;
+    KPM_CUDA(cudaDeviceSynchronize());
+    for (auto& o : w.cs)
+      if (&o != &cs) free_cols(o);
+    return KPM_OK;
+  };
+  auto alloc = [&]() -> kpm_status {
+    kpm_status a_ = dalloc((char**)&cs.tasks, tasks.size() * sizeof(ColsTask));
+    if (a_ == KPM_OK) a_ = dalloc(&cs.queue, (size_t)1);
+    if (a_ == KPM_OK && part) a_ = dalloc(&cs.part, part);
+    if (a_ != KPM_OK) free_cols(cs);
+    return a_;
+  };
+  if (part * sizeof(double) > ((size_t)64 << 20)) drop_others();
+  kpm_status sa = alloc();
+  if (sa == KPM_ENOMEM && drop_others() == KPM_OK) sa = alloc();
+  cs.S = S;
+  cs.R = R;
+  cs.fixq = fixq;
+  if (sa != KPM_OK) return sa == KPM_ENOMEM ? KPM_OK : sa;  // the solves in turn need none of it
   for (ColsTask& t : tasks)
     t.part = C > 1 ? (double*)((char*)cs.part + (size_t)t.part) : nullptr;
   KPM_CUDA(cudaMemcpyAsync(cs.tasks, tasks.data(), tasks.size() * sizeof(ColsTask),

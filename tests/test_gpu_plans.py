@@ -80,6 +80,30 @@ def test_alternating_start_blocks_keep_their_plans(K, user_first):
     assert np.abs(first[False] - O.moments_doubling(H, a, b, unit, M)[1]).max() <= 1e-10
 
 
+def test_kept_launches_give_way_without_memory(K):
+    """An allocation that fails while another (S, R) is kept: the kept one goes, the call
+    takes its form all the same, and the other one comes back when it is asked for."""
+    L, M, R = (10, 10, 10), 32, 4
+    with K.kpm_create_stencil(3, L) as h:
+        def call(S):
+            pv = K.kpm_moments(h, M, R, 6.1, 0.0, seed=3, S=S, per_vec=True)[1]
+            return pv, K.kpm_testing_last_step_form(h)
+
+        big, form = call(64)
+        assert form == "column strips"
+        want = call(32)
+        for after in range(3):
+            assert np.array_equal(call(64)[0], big)
+            K.kpm_testing_fail_allocations(after)
+            try:
+                pv, form = call(33 + after)      # a shape that is not kept
+            finally:
+                K.kpm_testing_fail_allocations(-1)
+            assert form == "column strips"
+            assert np.abs(pv - big[:(33 + after) * R]).max() <= 1e-13
+        assert np.array_equal(call(32)[0], want[0])
+
+
 @pytest.mark.parametrize("S", [2, 16])
 def test_large_lattice_beside_a_fixed_point_chain(K, S):
     """90,000 sites: a chain in fixed point (unit 2^-52), column tasks on the FP64 pipe."""
