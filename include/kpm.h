@@ -61,9 +61,11 @@ typedef enum {
 typedef enum { KPM_REAL = 0, KPM_COMPLEX = 1 } kpm_field;
 
 typedef enum {
-  KPM_FP64 = 0,               /* vectors, products and moment sums in FP64, or in
-                                 64-bit fixed point of FP64's accuracy where the
-                                 operator allows it (kpm_moments) */
+  KPM_FP64 = 0,               /* vectors, products and moment sums in FP64; calls on
+                                 a handle with library-made start blocks in 64-bit
+                                 fixed point of FP64's accuracy where the operator
+                                 allows it (kpm_moments; not the batch, the server,
+                                 kpm_moments_csr_noalloc or a user_v0) */
   KPM_FP32_VEC_FP64_MOM = 1   /* vectors stored/streamed and products in FP32;
                                  moment dot products summed in FP64 from short
                                  FP32 partial sums; bounds and DOS in FP64 */

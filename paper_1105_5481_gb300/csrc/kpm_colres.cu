@@ -562,6 +562,10 @@ int bulk_batch(int cpc, int block) {
 //     latency of a dependent step plus its work.  Measured: 2D L=32/64/80/96,
 //     R=8: 2.91/3.09/3.87/3.91; L=64, R=32: 4.85; complex 3D L=12/16, R=16:
 //     4.51/7.27; FP32 2D L=64/96, R=16: 3.14/3.30; complex 3D L=16, R=32: 3.25.
+//     (FP64 on the FP64 pipe; in fixed point the chain is up to 2.4 times as fast,
+//     median 1.7.  Of 160 FP64 shapes for which the column-resident form is chosen, M =
+//     64, the fixed-point chain is faster in nine, complex fields of 576 to 4,096
+//     rows with 8 to 64 columns, by 3 to 38 %.)
 double work_factor(bool cplx, bool fp32) {
   return (cplx ? (fp32 ? 1.2 : 3.9) : 1.0) * (fp32 ? 0.8 : 1.0);
 }

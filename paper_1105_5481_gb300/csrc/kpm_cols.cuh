@@ -41,9 +41,11 @@
 // Measured (FP32, 256 uneven 2D instances of 16..128 sites a side, 16 vectors):
 // 26.1 ms per batch against 38.7 for the global-memory form, whose products are
 // chains of L2 round trips; 2.6 us per product and column of 96 x 96 sites, of
-// which 1.1 the recursion, 0.8 the dot chains and 0.7 their reduction (each
-// left out in turn).  Bound by issue slots and the latency of the chains at
-// 16 warps per SM.
+// which 1.1 the recursion, 0.8 the dot chains and 0.7 their reduction (timed with
+// each left out in turn).  Bound by the latency of the chains at 16 warps per SM:
+// issue 47 % active; of 6.8 warps' cycles per issue 2.2 wait on fixed latencies, 2.2
+// at the barrier and 1.2 for shared memory.  A batch takes the form where it is
+// estimated faster (cols_faster in kpm_batch_api.cu).
 #pragma once
 
 #include "kpm_cols.h"

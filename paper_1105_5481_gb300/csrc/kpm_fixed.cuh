@@ -34,10 +34,11 @@
 //
 // An element takes one rounding of 2^-q / 2 per product where FP64 takes one of
 // about 2^-54 relative per term.  Error of the moments against 113-bit arithmetic,
-// over the FP64 pipe's: 0.91 to 0.98 on 2,000 to 16,000 sites (M = 256), 0.97 real
-// 2D N = 2^18, 1.03 complex 3D N = 2^18 (M = 64), where an FP64 result's own
-// rounding shows.  A real row has the fewest terms: at q = 51 it measured 0.6 to
-// 1.4, so real fields stay above (fixed_kind).  The dots are sums of exact
+// over the FP64 pipe's: 0.91 to 0.98 on 2,000 to 16,000 sites (M = 256), 0.93 to 1.02
+// up to 2^20 complex and 2^18 real sites (FIXED_MAX_N_REAL in kpm_api.cu), where an
+// FP64 result's own rounding shows.  Coefficients have the absolute unit 2^-56: one
+// far below the largest keeps fewer bits than in FP64, but moves H by no more than
+// the FP64 rounding of the largest does.  The dots are sums of exact
 // products likewise (<v_n|v_n> <= N bounds them), converted to FP64 once per
 // thread group.  A value past 2^61 by a 64th (the spectrum is not enclosed: then a
 // moment has left [-1, 1] as well) sets bit 3 of the call's flags; the moments that

@@ -32,7 +32,7 @@ cudaError_t launch_step_f32(bool stencil, bool cplx, StepMode mode, const StepAr
                             const LaunchCfg& cfg, cudaStream_t st);
 cudaError_t launch_step_f64(bool stencil, bool cplx, StepMode mode, const StepArgs& a,
                             const LaunchCfg& cfg, cudaStream_t st);
-// FP64 vectors of a stencil in 64-bit fixed point (kpm_fixed.cuh, a.fixq > 0):
+// FP64 vectors of a stencil or CSR operator in 64-bit fixed point (kpm_fixed.cuh, a.fixq > 0):
 // the step, its CTAs per SM, and the conversions of FP64 vectors (in place, to
 // the unit 2^-q) and scaled coefficients
 cudaError_t launch_step_i64(bool stencil, bool cplx, StepMode mode, const StepArgs& a, const LaunchCfg& cfg,
