@@ -852,11 +852,12 @@ kpm_status kpm_create_csr(int64_t n, const int64_t* rowptr, const int32_t* col, 
   if (e != cudaSuccess) { destroy_handle(h); return cuda_fail(e, "copy CSR"); }
   // Short rows: keep a padded ELL copy for the fused step (fixed trip count, no
   // row-pointer indirection).  Width = longest row rounded up to even, used when
-  // it is at most 8 and the padding at most doubles the stored entries.
+  // it is at most 8 and the padding at most doubles the stored entries (an operator
+  // without entries has nothing to pad: its scaled values are not allocated).
   int64_t wmax = 0;
   for (int64_t i = 0; i < n; ++i) wmax = std::max(wmax, rowptr[i + 1] - rowptr[i]);
   const int64_t W = std::max<int64_t>(2, (wmax + 1) / 2 * 2);
-  if (wmax <= 8 && n * W <= 2 * std::max<int64_t>(nnz, 1)) {
+  if (nnz > 0 && wmax <= 8 && n * W <= 2 * nnz) {
     // built on the device from the CSR arrays just copied (padding slots point
     // at the row itself with value 0); + 4 entries: the TMA-fed ELL step copies
     // the last tile in whole 16-byte units
