@@ -267,7 +267,6 @@ __global__ void __launch_bounds__(FIN_STEPS * 32) finalize_kernel(const double* 
 
 // ------------------------------------------------------------------ Gershgorin
 __device__ __forceinline__ double cabs2(double re, double im) {
-  if (im == 0.0) return fabs(re);
   // (hypot's scaling, half of its FP64 instructions, only where it is needed)
   const double m = fma(re, re, im * im);
   return m > 1e-280 && m < 1e280 ? sqrt(m) : hypot(re, im);
@@ -311,11 +310,11 @@ __global__ void gershgorin_stencil_kernel(bool cplx, int64_t n, StencilGeom g,
       if (L == 2 && per) {  // both bonds join the same pair: |H_ij| = |t_f + conj(t_b)|
         hopv(i, fr, fi);
         hopv(jb, br, bi);
-        rad += cabs2(fr + br, fi - bi);
+        rad += cplx ? cabs2(fr + br, fi - bi) : fabs(fr + br);
         continue;
       }
-      if (hasf) { hopv(i, fr, fi); rad += cabs2(fr, fi); }
-      if (hasb) { hopv(jb, br, bi); rad += cabs2(br, bi); }
+      if (hasf) { hopv(i, fr, fi); rad += cplx ? cabs2(fr, fi) : fabs(fr); }
+      if (hasb) { hopv(jb, br, bi); rad += cplx ? cabs2(br, bi) : fabs(br); }
       (void)jf;
     }
     lo = fmin(lo, center - rad);
@@ -349,7 +348,7 @@ __global__ void gershgorin_csr_kernel(bool cplx, int64_t n, const int64_t* __res
       const double re = cplx ? val[2 * k] : val[k];
       const double im = cplx ? val[2 * k + 1] : 0.0;
       if (col[k] == i) center += re;
-      else rad += cabs2(re, im);
+      else rad += cplx ? cabs2(re, im) : fabs(re);
     }
     lo = fmin(lo, center - rad);
     hi = fmax(hi, center + rad);
