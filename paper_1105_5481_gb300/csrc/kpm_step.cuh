@@ -404,6 +404,10 @@ struct StencilOp {
     const T d = HAS_DS ? ldg_scal(reinterpret_cast<const T*>(a.ds), i) : du;
     acc.axpy(d, xi);
     T fr[DIMS], fi[DIMS], br[DIMS], bi[DIMS];
+    auto cut = [&](int d2) {  // bonds past an open edge
+      if (!hf[d2]) { fr[d2] = T(0); fi[d2] = T(0); }
+      if (!hb[d2]) { br[d2] = T(0); bi[d2] = T(0); }
+    };
 #pragma unroll
     for (int d2 = 0; d2 < DIMS; ++d2) {
       if constexpr (HAS_HOP) {
@@ -423,19 +427,16 @@ struct StencilOp {
       } else {
         fr[d2] = hu_r; fi[d2] = hu_i; br[d2] = hu_r; bi[d2] = -hu_i;
       }
+      if constexpr (!RowAcc<CH>::kIssueBound) cut(d2);
     }
     // (the selects are worth a uniform branch only where issue is the limit)
-    bool edges = true;
     if constexpr (RowAcc<CH>::kIssueBound) {
-      edges = false;
+      bool edges = false;
 #pragma unroll
       for (int d2 = 0; d2 < DIMS; ++d2) edges |= a.geom.periodic[d2] == 0;
-    }
-    if (edges) {
+      if (edges) {
 #pragma unroll
-      for (int d2 = 0; d2 < DIMS; ++d2) {
-        if (!hf[d2]) { fr[d2] = T(0); fi[d2] = T(0); }
-        if (!hb[d2]) { br[d2] = T(0); bi[d2] = T(0); }
+        for (int d2 = 0; d2 < DIMS; ++d2) cut(d2);
       }
     }
     const size_t rowS = (size_t)a.G * CH::SC;
@@ -512,7 +513,11 @@ struct StencilOp {
 
   // Row i in natural order: coordinates decoded from the index by multiply-high
   // (2D 500 x 301 with an open edge, 16 FP32 columns, L2-resident: 7.9 -> 7.5 us
-  // per product against the divisions by a variable).
+  // per product against the divisions by a variable).  Not on the FP64 pipe, which
+  // bounds its step in any case: without the divisions its 2D kernels take 80 registers
+  // in place of 84, three CTAs then fit an SM, and those of the next step, launched
+  // early, fill the third places unevenly (real with on-site terms, M = 32: 300 x 250,
+  // 8 columns 273 us against 224; 600 x 600, 4 columns 488 against 447).
   __device__ __forceinline__ void apply(const StepArgs& a, int64_t i64, const T* __restrict__ Xc,
                                         const CH& xi, Row& acc, T hu_r, T hu_i, T du) const {
     const int i = (int)i64;
@@ -523,7 +528,10 @@ struct StencilOp {
     for (int d2 = 0; d2 < DIMS; ++d2) {
       const int L = a.geom.L[d2], s = a.geom.stride[d2];
       int x = rem;
-      if (d2 + 1 < DIMS) {
+      if constexpr (std::is_same<T, double>::value) {
+        x = rem % L;
+        rem /= L;
+      } else if (d2 + 1 < DIMS) {
         rem = (int)fdiv((unsigned)rem, a.geom.by[d2 < 2 ? d2 : 0]);
         x -= rem * L;
       }
