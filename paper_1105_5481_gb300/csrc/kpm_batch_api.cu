@@ -302,13 +302,15 @@ double makespan(std::vector<double> items, int m) {
 // sites with many vectors give the global-memory form enough CTAs to hide its round
 // trips, and the strips' second sweep for the dots then costs more than it saves:
 // 256 lattices of 32 x 32 with 32 vectors 2.06 ms (strips) against 1.66, of 16^3 7.64
-// against 5.09; 113 of 31 to 41 a side 3.72 against 3.51.  The estimates (microseconds per product, fitted
-// to 570 batches of 1 to 256 lattices of 6 to 128 (2D) or 4 to 24 (3D) a side with 4
-// to 32 FP32 vectors) are within 10 % (strips) and 15 % (global; lower by up to half
-// for power-of-two planes) of the measured times.  With 15 % to spare the strips are
-// taken in one of those batches where they are slower, by 5 %, and left in 13 where
-// they are faster, by 5 to 9 % in most.  FP64: both are bound by the FP64 pipe; its
-// instructions are counted.
+// against 5.09; 113 of 31 to 41 a side 3.72 against 3.51.  The estimates (microseconds
+// per product, fitted to 570 batches of 1 to 256 lattices of 6 to 128 (2D) or 4 to 24
+// (3D) a side with 4 to 32 FP32 vectors) are within 10 % (strips) and 15 % (global;
+// lower by up to half for power-of-two planes) of the measured times.  On those and 320
+// random batches the choice costs 0.24 % against the better form of each: the strips are
+// taken in 15 where they are slower, by up to 13 %, and left in 11 where they are faster,
+// by up to 18 % (16^3 with 8 vectors 49 %).  The line allows short runs little for the
+// launches: at 16 products 256 lattices of 32 x 32 stay global as at 64.  FP64: both are
+// bound by the FP64 pipe, whose instructions are counted; 0.2 % on 256 batches.
 bool cols_faster(kpm_batch_s* b, int C) {
   ColsPlan p;
   if (!plan_cols(b, C, &p)) return false;
@@ -338,8 +340,8 @@ bool cols_faster(kpm_batch_s* b, int C) {
     }
     global.push_back(us * (b->inst_tasks[i].M / 2));
   }
-  const double t_global = 140.0 + makespan(global, nglob);
-  if (!b->fp32) return 1.25 * (40.0 + 1.2 * p.us) <= t_global;
+  const double t_global = makespan(global, nglob);
+  if (!b->fp32) return 1.2 * p.us <= t_global + 100.0;
   for (const ColsTask& t : p.tasks) {
     const int64_t passes = t.lines > 0 ? (int64_t)(t.lines + t.spi - 1) / t.spi * t.geom.L[0]
                                        : (t.n + t.spi - 1) / t.spi;
@@ -351,7 +353,7 @@ bool cols_faster(kpm_batch_s* b, int C) {
                          : 0.22 + 0.017 * t.height + 0.071 * sites + sweeps * (0.49 + 0.011 * rows);
     strips.push_back(us * (t.M / 2));
   }
-  return 1.15 * (20.0 + makespan(strips, p.clusters)) <= t_global;
+  return 0.95 * makespan(strips, p.clusters) <= t_global + 20.0;
 }
 
 int cfg_clusters(kpm_batch_s* b, const BatchConfig& c) {
