@@ -75,8 +75,8 @@ BATCH_SOURCES = STEP_SOURCES + ["paper_1105_5481_gb300/csrc/kpm_batch.cuh",
 # capture (steady state of consecutive launches, caches not flushed between
 # them), keyed by workload and launch configuration, with the hash of the
 # kernel sources it was taken on; reported only while the hash matches.
-MEASURED_TRAFFIC = {"cubic_spin_L64": (347.65e6, "step", "153c8d82dff9087b"),
-                    "csr_spin_dilute_L160": (3394.51e6, "tma", "aa8b5b1661825794"),
+MEASURED_TRAFFIC = {"cubic_spin_L64": (347.99e6, "step", "350edef43a3ff8a2"),
+                    "csr_spin_dilute_L160": (3392.44e6, "tma", "fc38ab37d6c906c7"),
                     "batch_2d_256/C4/chunk2/clusters74/rt1/top0": (69.20e9, "batch", "f1a1fabd8beeef38"),
                     "batch_2d_256/C4/chunk4/clusters74/rt1/top0": (68.25e9, "batch", "f1a1fabd8beeef38"),
                     "batch_2d_256/C4/chunk2/clusters74/rt2/top8": (61.17e9, "batch", "f1a1fabd8beeef38"),
